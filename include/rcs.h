@@ -219,9 +219,10 @@ int rcs_plan_pass(const rcs_plan *plan, size_t i, int32_t *k, int32_t *targets, 
 
 /* Device time (ms) of the full-state passes of the last rcs_apply_circuit or
  * rcs_plan_run on this context (CUDA events around them on the context's stream;
- * the sub-state prefix and expansion are not included), and how many kernel
- * launches they took (a two-unitary round trip is one launch). Waits for those
- * passes to finish. */
+ * the sub-state prefix and expansion are not included), and how many passes they
+ * were (a two-unitary round trip counts once; passes chained in one launch count
+ * each, although the state makes one trip through HBM for all of them). Waits for
+ * those passes to finish. */
 int rcs_last_pass_timing(rcs_ctx *ctx, float *ms, int64_t *full_passes);
 
 /* Uploads the plan's pass table and matrices to the device of ctx (once per plan

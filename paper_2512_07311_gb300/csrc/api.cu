@@ -44,6 +44,7 @@ struct rcs_ctx {
     bool zero_pending = false;
     float2 *d_sub = nullptr;  // compact sub-state for the first passes of a run from |0...0>
     size_t sub_cap = 0;
+    uint32_t *d_chain = nullptr;  // chunk counters of chained tensor-core passes
     cudaEvent_t ev_full[2] = {nullptr, nullptr};  // around the full-state passes of the last run
     int64_t timed_passes = -1;
     std::string err;
@@ -407,7 +408,8 @@ int run_passes(rcs_ctx *c, const Plan &plan, const uint8_t *d_ops, bool from_zer
             c->sub_cap = bytes;
         }
         int fused = 0;
-        if (run_substages(plan, stages, c->psi, c->d_sub, d_ops, c->d_err, c->stream, &fused) != RCS_OK)
+        if (run_substages(plan, stages, c->psi, c->d_sub, d_ops, c->d_err, c->stream, &fused, c->d_chain) !=
+            RCS_OK)
             return fail(c, RCS_ERR_CUDA, "sub-state stages: " + take_launch_error());
         c->zero_pending = false;
         first = size_t(pre + fused);
@@ -416,8 +418,8 @@ int run_passes(rcs_ctx *c, const Plan &plan, const uint8_t *d_ops, bool from_zer
     }
     cudaEventRecord(c->ev_full[0], c->stream);
     int64_t launches = 0;
-    if (launch_pass_range(plan, c->psi, c->n, first, plan.passes.size(), 0, d_ops, c->d_err, c->stream, &launches) !=
-        RCS_OK)
+    if (launch_pass_range(plan, c->psi, c->n, first, plan.passes.size(), 0, d_ops, c->d_err, c->stream, &launches,
+                          c->d_chain) != RCS_OK)
         return fail(c, RCS_ERR_CUDA, "launch of a full-state pass failed: " + take_launch_error());
     cudaEventRecord(c->ev_full[1], c->stream);
     c->timed_passes = launches;
@@ -475,18 +477,19 @@ int plan_fresh_circuit(int n, const std::vector<HostGate> &gates, const rcs_opts
 
 Pass substate_pass(const Pass &p, uint64_t T) { return compact_pass(p, T); }
 
-int launch_plan_pass(void *psi, int n, const Pass &p, const uint8_t *ops, int *d_err, void *stream, bool tf32) {
+int launch_plan_pass(void *psi, int n, const Pass &p, const uint8_t *ops, int *d_err, void *stream, bool tf32,
+                     bool backwards) {
     switch (p.kind) {
         case PASS_1Q:
         case PASS_2Q: return launch_pass_plain(psi, n, p, stream);
         case PASS_SIMT: return launch_pass_simt(psi, n, p, ops, stream);
-        case PASS_TC: return launch_pass_tc(psi, n, p, ops, d_err, stream, tf32);
+        case PASS_TC: return launch_pass_tc(psi, n, p, ops, d_err, stream, tf32, backwards);
         default: return RCS_ERR_ARG;
     }
 }
 
 int run_substages(const Plan &plan, const std::vector<SubStage> &stages, void *psi, void *sub, const uint8_t *d_ops,
-                  int *d_err, void *stream, int *fused) {
+                  int *d_err, void *stream, int *fused, uint32_t *chain_sync) {
     const bool tf32 = plan_tf32(plan);
     *fused = 0;
     uint8_t *buf = static_cast<uint8_t *>(sub);
@@ -510,7 +513,7 @@ int run_substages(const Plan &plan, const std::vector<SubStage> &stages, void *p
         }
         int64_t launches = 0;
         if (launch_pass_range(plan, next, m, size_t(st.first), size_t(st.first + st.count), st.tmask, d_ops, d_err,
-                              stream, &launches) != RCS_OK)
+                              stream, &launches, chain_sync) != RCS_OK)
             return RCS_ERR_CUDA;
         cur = next;
         cur_mask = st.tmask;
@@ -530,15 +533,45 @@ bool plan_pairs_at(const Plan &plan, size_t i, size_t end, int n) {
 }
 
 int launch_pass_range(const Plan &plan, void *psi, int n, size_t first, size_t end, uint64_t T, const uint8_t *d_ops,
-                      int *d_err, void *stream, int64_t *launches) {
+                      int *d_err, void *stream, int64_t *launches, uint32_t *chain_sync) {
     const bool tf32 = plan_tf32(plan);
+    const bool images = plan.tc_offset.size() == plan.passes.size();
+    // chains of passes: the split looks at targets only, so the matrices are left out
+    std::vector<Pass> shape;
+    std::vector<int> chain;
+    if (chain_sync && images && !plan.pairs) {
+        for (size_t i = first; i < end; ++i) {
+            const Pass &p = plan.passes[i];
+            Pass q;
+            q.kind = plan.tc_offset[i] >= 0 ? p.kind : PASS_SIMT;
+            q.k = p.k;
+            for (int j = 0; j < p.k; ++j) q.t[j] = T ? std::popcount(T & ((1ull << p.t[j]) - 1ull)) : p.t[j];
+            shape.push_back(std::move(q));
+        }
+        chain = tc_chain_lengths(shape, n, tf32);
+    }
     Pass c0, c1;  // targets renumbered into the sub-state
     auto at = [&](size_t i, Pass &tmp) -> const Pass & {
         if (!T) return plan.passes[i];
         tmp = compact_pass(plan.passes[i], T);
         return tmp;
     };
-    for (size_t i = first; i < end;) {
+    bool backwards = false;  // launches walk the state in turn from either end: L2 still holds the last part
+    for (size_t i = first; i < end; backwards = !backwards) {
+        if (!chain.empty() && chain[i - first] > 1) {
+            const int count = chain[i - first];
+            const Pass *ps[8];
+            const void *ops[8];
+            for (int j = 0; j < count; ++j) {
+                ps[j] = &shape[i - first + size_t(j)];
+                ops[j] = d_ops + plan.tc_offset[i + size_t(j)];
+            }
+            if (launch_chain_tc(psi, n, ps, ops, count, chain_sync, d_err, stream, backwards) != RCS_OK)
+                return RCS_ERR_CUDA;
+            *launches += count;
+            i += size_t(count);
+            continue;
+        }
         const Pass &p = at(i, c0);
         if (plan_pairs_at(plan, i, end, n) && plan.pair_offset.size() == plan.passes.size() &&
             plan.pair_offset[i] >= 0 && plan.pair_offset[i + 1] >= 0) {
@@ -550,10 +583,8 @@ int launch_pass_range(const Plan &plan, void *psi, int n, size_t first, size_t e
             i += 2;
             continue;
         }
-        const uint8_t *ops = plan.tc_offset.size() == plan.passes.size() && plan.tc_offset[i] >= 0
-                                 ? d_ops + plan.tc_offset[i]
-                                 : nullptr;
-        if (launch_plan_pass(psi, n, p, ops, d_err, stream, tf32) != RCS_OK) return RCS_ERR_CUDA;
+        const uint8_t *ops = images && plan.tc_offset[i] >= 0 ? d_ops + plan.tc_offset[i] : nullptr;
+        if (launch_plan_pass(psi, n, p, ops, d_err, stream, tf32, backwards) != RCS_OK) return RCS_ERR_CUDA;
         ++*launches;
         ++i;
     }
@@ -614,6 +645,7 @@ void rcs_destroy(rcs_ctx *c) {
     cudaFree(c->d_order);
     cudaFree(c->d_ops);
     cudaFree(c->d_sub);
+    cudaFree(c->d_chain);
     if (c->ev_full[0]) cudaEventDestroy(c->ev_full[0]);
     if (c->ev_full[1]) cudaEventDestroy(c->ev_full[1]);
     cudaSetDevice(prev);
@@ -677,6 +709,9 @@ int rcs_create(const rcs_grid *grid, const rcs_opts *opts, rcs_ctx **out) {
         return rc;
     if ((rc = alloc(reinterpret_cast<void **>(&c->total), 8, "total")) != RCS_OK) return rc;
     if ((rc = alloc(reinterpret_cast<void **>(&c->d_err), sizeof(int), "error word")) != RCS_OK) return rc;
+    if (o.precision == RCS_PREC_BF16X3)
+        if (const size_t cb = tc_chain_sync_bytes(c->n); cb > 0)
+            if ((rc = alloc(reinterpret_cast<void **>(&c->d_chain), cb, "chain counters")) != RCS_OK) return rc;
     if (cudaMemset(c->d_err, 0, sizeof(int)) != cudaSuccess || cudaEventCreate(&c->ev_full[0]) != cudaSuccess ||
         cudaEventCreate(&c->ev_full[1]) != cudaSuccess) {
         std::string msg = std::string("initialisation: ") + cudaGetErrorString(cudaGetLastError());

@@ -136,11 +136,13 @@ size_t substage_bytes(const std::vector<SubStage> &stages);
 // sub-state, its passes, an expansion into the next sub-state, ..., and either an
 // expansion into psi or, when the next pass can read a sub-state, that pass taking the
 // last sub-state as input (*fused = 1: the caller resumes one pass later). `sub` holds
-// substage_bytes(stages). Asynchronous; launch error text kept.
+// substage_bytes(stages). chain_sync: scratch for chains (launch_pass_range), or null.
+// Asynchronous; launch error text kept.
 int run_substages(const Plan &plan, const std::vector<SubStage> &stages, void *psi, void *sub,
-                  const uint8_t *d_ops, int *d_err, void *stream, int *fused);
+                  const uint8_t *d_ops, int *d_err, void *stream, int *fused, uint32_t *chain_sync);
 // Launches one pass of a plan on a 2^n-amplitude state (ops: its operand image, if any).
-int launch_plan_pass(void *psi, int n, const Pass &p, const uint8_t *ops, int *d_err, void *stream, bool tf32);
+int launch_plan_pass(void *psi, int n, const Pass &p, const uint8_t *ops, int *d_err, void *stream, bool tf32,
+                     bool backwards = false);
 int launch_pass_plain(void *psi, int n, const Pass &p, void *stream);
 // Fused FP32 SIMT pass of width p.k = 1..kSimtKMax. Widths up to kSimtParamK carry U in
 // the kernel parameters (ops unused); wider ones read it from ops, the device copy of
@@ -156,7 +158,10 @@ int simt_prepare_device();
 // launch_pass_tc calls it, and a caller about to capture a graph calls it first.
 int tc_prepare_device();
 // tf32: the TF32x3 kernel (operand image from tc_build_ops(p, img, true)), else BF16x3.
-int launch_pass_tc(void *psi, int n, const Pass &p, const void *d_ops, int *d_err, void *stream, bool tf32);
+// backwards: walk the state from its end (a pass that follows a forward one then finds the
+// end of the state in L2; a hint, ignored by the memory-order kernel).
+int launch_pass_tc(void *psi, int n, const Pass &p, const void *d_ops, int *d_err, void *stream, bool tf32,
+                   bool backwards = false);
 // The same pass reading its input from a sub-state instead of psi: the state is |0> on
 // the qubits outside tmask, and sub holds its amplitudes with those qubits at 0 at their
 // compact index; the pass writes the whole 2^n state to psi (an expansion and a pass in
@@ -164,6 +169,15 @@ int launch_pass_tc(void *psi, int n, const Pass &p, const void *d_ops, int *d_er
 bool tc_pass_takes_substate(const Pass &p, int n);
 int launch_pass_tc_from_sub(void *psi, int n, const Pass &p, const void *d_ops, int *d_err, void *stream, bool tf32,
                             const void *sub, uint64_t tmask);
+
+// Chains: 2 or 3 consecutive BF16x3 tensor-core passes in one launch, the state making one trip
+// through HBM (k_tc.cu). tc_chain_lengths splits a sequence of passes on n qubits: entry i
+// is the number of passes of the group that starts at i. `sync` is scratch of
+// tc_chain_sync_bytes(n) device bytes (0: no chains at that size), cleared by each launch.
+size_t tc_chain_sync_bytes(int n);
+std::vector<int> tc_chain_lengths(const std::vector<Pass> &passes, int n, bool tf32);
+int launch_chain_tc(void *psi, int n, const Pass *const *p, const void *const *d_ops, int count, uint32_t *sync,
+                    int *d_err, void *stream, bool backwards);
 
 // Test hook of the tensor-core kernels' bounded waits (process-wide): the wait limit and
 // the tile (of CTA 0) whose MMAs are skipped, as every launch reads them, and the setter.
@@ -215,9 +229,10 @@ int launch_pair_tc(void *psi, int n, const Pass &p1, const Pass &p2, const void 
 bool plan_pairs_at(const Plan &plan, size_t i, size_t end, int n);
 // Launches passes [first, end) of a plan on the 2^n-amplitude state psi, their targets
 // renumbered into the sub-state of mask T when T != 0; consecutive tensor-core passes
-// share a round trip where plan_pairs_at says so. *launches counts kernel launches.
+// share a round trip where plan_pairs_at says so, and run as chains (tc_chain_lengths) when
+// chain_sync is given. *launches counts passes (a two-unitary round trip once).
 int launch_pass_range(const Plan &plan, void *psi, int n, size_t first, size_t end, uint64_t T, const uint8_t *d_ops,
-                      int *d_err, void *stream, int64_t *launches);
+                      int *d_err, void *stream, int64_t *launches, uint32_t *chain_sync);
 
 // Sampler / readout (k_sample.cu)
 // to_stored: caller basis index -> stored index (the state's qubit layout). Blocks are

@@ -43,7 +43,9 @@
 
 #include <algorithm>
 #include <atomic>
+#include <bit>
 #include <cstring>
+#include <vector>
 
 #include "dev_common.cuh"
 #include "internal.h"
@@ -52,12 +54,26 @@
 
 namespace rcs {
 
+// One pass as the kernel reads it. Slice-order addressing is in bytes: a tile's base | a
+// slice row's base | a local amplitude's offset; the offsets are constant operands of the
+// address adds.
+struct TcPass {
+    const uint4 *ops;    // B operand images in their shared-memory layout (BF16: 64 KB, TF32: 96 KB)
+    uint64_t joff[32];   // local amplitude j < 32 (j's bits on targets 0..4)
+    uint64_t joff5;      // local amplitude bit 5 (target 5)
+    uint64_t coff[8];    // copy c of a loader's unit (see the slice-order loader)
+    int t[tc::K];        // ascending targets
+    int8_t rpos[7];      // index bit of slice row bit i: the 7 lowest non-target qubits
+    int8_t tpos[32];     // index bit of tile number bit i: the other qubits (-1: none), those of the
+                         // chunk first (a chain), else ascending
+};
+
+template <int kPasses>
 struct TcArgs {
     float2 *psi;
-    const uint4 *ops;  // B operand images in their shared-memory layout (BF16: 64 KB, TF32: 96 KB)
     int *err;
     uint32_t tiles;
-    int t[tc::K];      // ascending targets
+    TcPass pass[kPasses];
     uint64_t vmask;    // qubits varying inside a tile: the targets and the 7 lowest other qubits
     int r;             // qubits 0 .. r-1 all lie in vmask (r >= 7): contiguous runs of 2^r amplitudes
     // Input from a sub-state (kSub): the state is |0> on the qubits outside `tmask`, and
@@ -67,6 +83,13 @@ struct TcArgs {
     uint64_t tmask;
     long long wait_cycles;  // limit of every wait (SM clock cycles)
     int skip_tile;          // test hook: CTA 0 issues no MMAs for its tile skip_tile (-1: none)
+    uint32_t flip;          // XORed into the tile numbers: 0, or tiles - 1 to walk the state backwards
+    uint32_t depth;         // slice order: units a loader warp keeps in flight or in conversion, 2..kSlots
+    // Chain (kChain): see the comment at k_fused_tc.
+    int npass;              // passes of the chain, 2..kChainMax
+    int clog;               // log2 of the tiles in a chunk
+    uint32_t window;        // chunks a pass may be ahead of the next one
+    uint32_t *sync;         // [0]: launch-wide abort word; [1 + p * chunks + c]: tiles of chunk c that pass p has stored
 };
 
 // Position of compact tile index c in the memory-order stage: XOR-swizzles bits
@@ -84,10 +107,32 @@ __device__ __forceinline__ uint32_t swz(uint32_t c) { return c ^ ((c >> 6) & 15u
 // kTf32 = true: TF32 split of the complex block form (48 MMAs of K = 8 per tile).
 // kSub (slice order only): the loads come from the sub-state a.sub instead of psi (see
 // TcArgs), so the pass both expands the sub-state and applies its unitary.
-template <bool kStaged, bool kTf32, bool kSub>
-__global__ void __launch_bounds__(tc::kThreads, 1) k_fused_tc(const __grid_constant__ TcArgs a) {
+// kChain (slice order, BF16 only): 2 or 3 consecutive passes in one launch, with one trip of the
+// state through HBM. A chunk is the set of amplitudes that differ only in the chain's
+// targets and the lowest qubits, so every pass maps a chunk to itself. CTA b works on pass
+// b mod npass; the CTAs of a pass take its tiles in chunk order, and a pass starts a chunk
+// once the pass before it has stored all of it. A chunk then still sits in L2: with chunks
+// of 4 to 16 MB and a window of 64 to 80 MB between passes, the first pass reads HBM, the
+// last one's stores go back to it, and all else runs at L2's rate: at 27 qubits a pair of
+// passes takes 458 us against 2 x 323 one after the other (where HBM runs at its peak), and
+// the SM's own pipeline (2.1 us per tile: 1.5 without any copies and stores) is the bound.
+// TF32x3 tiles take the SM longer than HBM needs for them, and chains of them measured slower. Two more warps keep the
+// order, so that the loaders and the epilogue never wait for L2:
+//   warp 17 polls the chunk counters of the passes before and after this CTA's, and tells
+//           the loaders in shared memory how many chunks they may start (the next pass holds
+//           this one back to `window` chunks ahead of it, so a chunk is read while in L2);
+//   warp 18 publishes: when all epilogue warps have stored their part of the CTA's tiles of
+//           a chunk it fences and adds their number to the chunk's counter.
+// A loader never blocks on a chunk while a tile of its CTA is unconverted, and a wait of
+// (pass p, chunk c) is on (p - 1, c) or (p + 1, c - window) only: with all CTAs resident
+// (a cooperative launch) the schedule cannot deadlock.
+template <bool kStaged, bool kTf32, bool kSub, bool kChain>
+__global__ void __launch_bounds__(kChain ? tc::kChainThreads : tc::kThreads, 1)
+    k_fused_tc(const __grid_constant__ TcArgs<kChain ? tc::kChainMax : 1> a) {
     static_assert(!(kStaged && kSub), "the sub-state input has a slice-order loader only");
+    static_assert(!kChain || (!kStaged && !kSub && !kTf32), "a chain runs BF16 passes in slice order");
     using namespace tc;
+    constexpr int kThreads = kChain ? tc::kChainThreads : tc::kThreads;
     using L = Layout<kTf32>;
     extern __shared__ uint8_t smem_raw[];
     uint8_t *sm = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -114,17 +159,25 @@ __global__ void __launch_bounds__(tc::kThreads, 1) k_fused_tc(const __grid_const
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const long long lim = a.wait_cycles;
+    // chain: this CTA's pass, its number among that pass's CTAs, and their count
+    const uint32_t pidx = kChain ? blockIdx.x % uint32_t(a.npass) : 0u;
+    const uint32_t cta = kChain ? blockIdx.x / uint32_t(a.npass) : blockIdx.x;
+    const uint32_t ctas = kChain ? (gridDim.x - pidx + uint32_t(a.npass) - 1u) / uint32_t(a.npass) : gridDim.x;
+    const TcPass &ps = a.pass[pidx];
+    // chain: chunks the loaders may start, and per epilogue warp the chunks it has stored its part of
+    volatile uint32_t *chunk_limit = reinterpret_cast<volatile uint32_t *>(sm + L::kMisc + 8);
+    volatile uint32_t *chunk_out = reinterpret_cast<volatile uint32_t *>(sm + L::kMisc + 16);
     int t[K];
 #pragma unroll
-    for (int i = 0; i < K; ++i) t[i] = a.t[i];
+    for (int i = 0; i < K; ++i) t[i] = ps.t[i];
 
     // ---- set-up: operand image, offset table, barriers, tensor memory
     {
         uint4 *dst = reinterpret_cast<uint4 *>(sm);
-        for (int i = threadIdx.x; i < L::kBBytes / 16; i += kThreads) dst[i] = a.ops[i];
+        for (int i = threadIdx.x; i < L::kBBytes / 16; i += kThreads) dst[i] = ps.ops[i];
         const uint64_t V = a.vmask;
         auto cpos = [&](int qb) { return __popcll(V & ((1ull << qb) - 1ull)); };  // compact position of qubit qb
-        if (threadIdx.x < D) {
+        if ((kStaged || kSub) && threadIdx.x < D) {
             uint64_t o = 0;
             uint32_t c = 0;
 #pragma unroll
@@ -159,7 +212,7 @@ __global__ void __launch_bounds__(tc::kThreads, 1) k_fused_tc(const __grid_const
                 hi_off[threadIdx.x] = cpos_sub;  // hi_off serves the memory-order variant only
             }
         }
-        if (threadIdx.x < M) {
+        if (kStaged && threadIdx.x < M) {
             // slice bit k sits on the k-th lowest qubit that is not a target
             uint32_t c = 0;
             int k = 0;
@@ -185,6 +238,10 @@ __global__ void __launch_bounds__(tc::kThreads, 1) k_fused_tc(const __grid_const
                 mbar_init(bar_sfree(b), kEpiWarps);
             }
             *abort_flag = 0;
+            if constexpr (kChain) {
+                *chunk_limit = 0;
+                for (int e = 0; e < kEpiWarps; ++e) chunk_out[e] = 0;
+            }
             asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         }
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -200,7 +257,7 @@ __global__ void __launch_bounds__(tc::kThreads, 1) k_fused_tc(const __grid_const
     }
     const uint32_t tmem = *tmem_slot;
     const uint32_t ntile = a.tiles;
-    const uint32_t my_tiles = blockIdx.x < ntile ? (ntile - 1 - blockIdx.x) / gridDim.x + 1 : 0;
+    const uint32_t my_tiles = cta < ntile ? (ntile - 1 - cta) / ctas + 1 : 0;
 
     // Tensor-memory plan. BF16: two buffers of {D: 128 cols, A_hi: 64, A_lo: 64} at
     // column 256 b. TF32: D double-buffered at column 128 b (Re outputs in its first 64
@@ -266,6 +323,23 @@ __global__ void __launch_bounds__(tc::kThreads, 1) k_fused_tc(const __grid_const
 
     const uint32_t rmask = (1u << a.r) - 1u;
     const uint32_t stage0_u32 = smem_u32(sm + L::kStage0);
+    // Slice order: the byte offset of slice row r of a tile, and of a tile. Lane l deposits
+    // bit l of the tile number and the warp combines the 32 parts with two reductions.
+    auto row_bytes = [&](int r) {
+        uint64_t o = 0;
+#pragma unroll
+        for (int i = 0; i < 7; ++i)
+            if ((r >> i) & 1) o |= 8ull << ps.rpos[i];
+        return o;
+    };
+    const int tpos = ps.tpos[lane];
+    const uint64_t tbit = tpos >= 0 ? 8ull << tpos : 0ull;
+    auto tile_bytes = [&](uint32_t tile) {
+        const bool on = (tile >> lane) & 1u;
+        const uint32_t lo = __reduce_or_sync(0xffffffffu, on ? uint32_t(tbit) : 0u);
+        const uint32_t hi = __reduce_or_sync(0xffffffffu, on ? uint32_t(tbit >> 32) : 0u);
+        return (uint64_t(hi) << 32) | lo;
+    };
     if (warp < kLoaderWarps && !kStaged) {
         // ---------------------------------------------------------------- loaders (slice order)
         const int q = warp & 3, h = warp >> 2;  // TMEM lane quarter, amplitude half
@@ -322,10 +396,9 @@ __global__ void __launch_bounds__(tc::kThreads, 1) k_fused_tc(const __grid_const
                         put16(abase_of(b, h) + (uint32_t(32 * q) << 16), acol_in(h, ch), zero16);
             asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
         }
-        auto issue = [&](uint32_t i, int b) {
-            const uint64_t tile = uint64_t(blockIdx.x) + uint64_t(i) * gridDim.x;
-            const uint64_t base = slice_base(tile * M + srow, t);
-            if constexpr (kSub) {
+        if constexpr (kSub) {
+            auto issue = [&](uint32_t i, int b) {
+                const uint64_t tile = uint64_t(blockIdx.x) + uint64_t(i) * gridDim.x;
                 // a slice with a qubit outside the sub-state set is all zeros; otherwise amplitude
                 // j is at compact index (row and tile parts of the slice) | pext(off[j]) unless
                 // off[j] leaves the sub-state. Zeros come from copies of 0 source bytes (no read):
@@ -352,40 +425,170 @@ __global__ void __launch_bounds__(tc::kThreads, 1) k_fused_tc(const __grid_const
                     asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(dst), "l"(src), "r"(nbytes)
                                  : "memory");
                 }
-            } else {
-#pragma unroll 8
-                for (int jj = 0; jj < 32; ++jj) {
-                    const int j = 32 * h + jj;
-                    const float2 *src = a.psi + (base | off[j]);
-                    const uint32_t dst = stage0_u32 + uint32_t(b * kStageBytes + (j * M + srow) * 8);
-                    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(dst), "l"(src) : "memory");
+                asm volatile("cp.async.commit_group;" ::: "memory");
+            };
+            if (my_tiles > 0) issue(0, 0);
+            if (my_tiles > 1) issue(1, 1);
+            for (uint32_t i = 0; i < my_tiles; ++i) {
+                const int b = i & 1;
+                if (i + 1 < my_tiles) asm volatile("cp.async.wait_group 1;" ::: "memory");
+                else asm volatile("cp.async.wait_group 0;" ::: "memory");
+                if (!wait_a_free(i, h)) break;
+                tc_fence_after();
+                const float2 *stage = reinterpret_cast<const float2 *>(sm + L::kStage0 + b * kStageBytes);
+                const uint32_t abase = abase_of(b, h) + (uint32_t(32 * q) << 16);
+#pragma unroll
+                for (int ch = 0; ch < 2; ++ch) {  // 16 amplitudes (TMEM columns) at a time
+                    if (((jnz >> (32 * h + 16 * ch)) & 0xffffull) == 0) continue;  // zero columns
+                    float2 v[16];
+#pragma unroll
+                    for (int jj = 0; jj < 16; ++jj) v[jj] = stage[(32 * h + 16 * ch + jj) * M + srow];
+                    put16(abase, acol_in(h, ch), v);
                 }
+                asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(bar_full_h(b, h));
+                if (i + 2 < my_tiles) issue(i + 2, b);
             }
-            asm volatile("cp.async.commit_group;" ::: "memory");
-        };
-        if (my_tiles > 0) issue(0, 0);
-        if (my_tiles > 1) issue(1, 1);
-        for (uint32_t i = 0; i < my_tiles; ++i) {
-            const int b = i & 1;
-            if (i + 1 < my_tiles) asm volatile("cp.async.wait_group 1;" ::: "memory");
-            else asm volatile("cp.async.wait_group 0;" ::: "memory");
-            if (!wait_a_free(i, h)) break;
-            tc_fence_after();
-            const float2 *stage = reinterpret_cast<const float2 *>(sm + L::kStage0 + b * kStageBytes);
-            const uint32_t abase = abase_of(b, h) + (uint32_t(32 * q) << 16);
-#pragma unroll
-            for (int ch = 0; ch < 2; ++ch) {  // 16 amplitudes (TMEM columns) at a time
-                if (((jnz >> (32 * h + 16 * ch)) & 0xffffull) == 0) continue;  // kSub: zero columns
-                float2 v[16];
-#pragma unroll
-                for (int jj = 0; jj < 16; ++jj) v[jj] = stage[(32 * h + 16 * ch + jj) * M + srow];
-                put16(abase, acol_in(h, ch), v);
+        } else {
+            // A warp's part of a tile is its 32 slices x 32 amplitudes, moved in two units of 16
+            // amplitudes (4 KB) through the warp's own ring of kSlots stage slots: while a unit is
+            // converted, up to kSlots - 1 later ones are in flight, and each slot is filled again as
+            // soon as it is converted.
+            // Copies are 16 bytes wide and bypass L1. For each pair of amplitudes (j = 2 jp, 2 jp + 1,
+            // which differ in the lowest target) the 64 values of the warp are one 512-byte block in
+            // the order of their index bits: bit tb is the lowest target (bit 5 if that lies above bit
+            // 4), the others are the slice bits. So the lanes of a copy go up both in memory and in the
+            // stage, and with one target below bit 6 a copy reads 512 contiguous bytes. (Where a
+            // 32-byte sector or a line went to two places of the stage, L2 was read twice as often: 33
+            // against 23 us a pass at 23 qubits with the lowest target on bit 1.) With tb = 2 or 3 the
+            // blocks' lines 1 and 3 have their halves or sectors swapped, which keeps the reads below
+            // on different banks. With targets on bits 0 and 1 (quad) a sector holds amplitudes 4 i ..
+            // 4 i + 3 of one slice: neighbouring lanes then take its two halves, and the two halves of
+            // the warp's slices are two blocks. The 8-byte copies that came before went through L1 (a second pass of
+            // every byte over its data pipe) and re-read a 64-entry offset table from shared memory per
+            // amplitude: that pipe was 85% busy and a tile took 2.57 us per SM from L2.
+            constexpr uint32_t kSlots = L::kSlots;
+            const int tb = t[0] < 5 ? t[0] : 5;
+            const bool quad = t[0] == 0 && t[1] == 1;
+            const uint32_t swl = (tb == 2 || tb == 3) ? ((uint32_t(lane) >> 3) & 1u) << (tb - 1) : 0u;
+            // a lane's first value: its slice (2 lane without bit tb) and amplitude of the pair
+            const int cs0 = quad ? lane >> 1 : ((2 * lane) & ((1 << tb) - 1)) | (((2 * lane) >> (tb + 1)) << tb);
+            const uint64_t cj0 = quad ? ((lane & 1) ? ps.joff[2] : 0ull) : (((2 * lane) >> tb) & 1) ? ps.joff[1] : 0ull;
+            const uint64_t cbase = row_bytes(32 * q + cs0) + (h ? ps.joff5 : 0ull) + cj0;
+            const uint32_t ring = uint32_t(warp) * kSlots * kSlotBytes;
+            const uint32_t cdst = stage0_u32 + ring + ((uint32_t(lane) ^ swl) << 4);
+            // where this thread's slice sits in a block: j even, j odd
+            uint32_t rx = ((uint32_t(lane) >> tb) << (tb + 1)) | (uint32_t(lane) & ((1u << tb) - 1u));
+            if (tb == 2 || tb == 3) rx ^= ((rx >> 4) & 1u) << tb;
+            uint32_t rd0 = ring + rx * 8u, rd1 = rd0 ^ (8u << tb);
+            if (quad) {  // j = 0, 1 and j = 2, 3 of a slice are the 32 bytes there
+                rd0 = ring + (uint32_t(lane) & 15u) * 32u + (uint32_t(lane) >> 4) * 512u;
+                rd1 = rd0 + 16u;
             }
-            asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(bar_full_h(b, h));
-            if (i + 2 < my_tiles) issue(i + 2, b);
+            // chain: whether tile i's chunk may be started; waits for it if asked to (false: abort)
+            uint32_t chunks_open = 0;
+            auto open = [&](uint32_t i, bool block) {
+                if constexpr (!kChain) return true;
+                const uint32_t c = (cta + i * ctas) >> a.clog;
+                if (c < chunks_open) return true;
+                const long long t0 = clock64();
+                for (;;) {
+                    uint32_t v = lane == 0 ? *chunk_limit : 0u;
+                    v = __shfl_sync(0xffffffffu, v, 0);
+                    if (c < v) {
+                        chunks_open = v;
+                        __threadfence_block();  // the copies below come after the counters that warp 17 saw
+                        return true;
+                    }
+                    if (!block) return false;
+                    int stop = 0;
+                    if (lane == 0) {
+                        if (*abort_flag) stop = 1;
+                        else if (clock64() - t0 > lim) *abort_flag = stop = 1;
+                    }
+                    if (__shfl_sync(0xffffffffu, stop, 0)) return false;
+                    __nanosleep(64);
+                }
+            };
+
+            const uint32_t units = 2 * my_tiles;
+            uint32_t issued = 0, wslot = 0, rslot = 0;
+            const uint8_t *src = nullptr;  // the tile being issued
+            // issues units up to the ring's size past unit u; unit u itself must go (false: abort)
+            auto top_up = [&](uint32_t u) {
+                while (issued < units && issued < u + a.depth) {
+                    if (!(issued & 1u)) {
+                        // every earlier tile is converted if this is unit u, so waiting for the
+                        // tile's chunk holds up nothing that another CTA needs
+                        if (!open(issued >> 1, issued == u)) return issued != u;
+                        src = reinterpret_cast<const uint8_t *>(a.psi) + (cbase | tile_bytes((cta + (issued >> 1) * ctas) ^ a.flip));
+                    }
+                    const uint8_t *from = src + ((issued & 1u) ? ps.joff[16] : 0ull);
+                    const uint32_t to = cdst + wslot * kSlotBytes;
+#pragma unroll
+                    for (int jp = 0; jp < 8; ++jp)
+                        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(to + uint32_t(jp) * 512u),
+                                     "l"(from + ps.coff[jp])
+                                     : "memory");
+                    asm volatile("cp.async.commit_group;" ::: "memory");
+                    ++issued;
+                    if (++wslot == kSlots) wslot = 0;
+                }
+                return true;
+            };
+            bool ok = true;
+            for (uint32_t i = 0; i < my_tiles && ok; ++i) {
+                const int b = i & 1;
+                const uint32_t abase = abase_of(b, h) + (uint32_t(32 * q) << 16);
+#pragma unroll
+                for (int ch = 0; ch < 2; ++ch) {
+                    const uint32_t u = 2 * i + uint32_t(ch);
+                    __syncwarp();  // every lane has read the slot that is filled next
+                    if (!(ok = top_up(u))) break;
+                    const uint32_t later = issued - u - 1;  // units in flight behind this one
+                    if (later >= kSlots - 1) asm volatile("cp.async.wait_group %0;" ::"n"(kSlots - 1) : "memory");
+                    else if (later == 3) asm volatile("cp.async.wait_group 3;" ::: "memory");
+                    else if (later == 2) asm volatile("cp.async.wait_group 2;" ::: "memory");
+                    else if (later == 1) asm volatile("cp.async.wait_group 1;" ::: "memory");
+                    else asm volatile("cp.async.wait_group 0;" ::: "memory");
+                    __syncwarp();  // the warp's copies, made by other lanes, are visible to this one
+                    if (ch == 0) {
+                        if (!(ok = wait_a_free(i, h))) break;
+                        tc_fence_after();
+                    }
+                    const uint8_t *slot = sm + L::kStage0 + rslot * kSlotBytes;
+                    if (++rslot == kSlots) rslot = 0;
+                    float2 v[16];
+                    if (quad) {
+#pragma unroll
+                        for (int jj = 0; jj < 16; jj += 2) {
+                            const float4 w =
+                                *reinterpret_cast<const float4 *>(slot + ((jj & 2) ? rd1 : rd0) + (jj / 4) * 1024);
+                            v[jj] = make_float2(w.x, w.y);
+                            v[jj + 1] = make_float2(w.z, w.w);
+                        }
+                    } else if (tb == 0) {
+#pragma unroll
+                        for (int jj = 0; jj < 16; jj += 2) {
+                            const float4 w = *reinterpret_cast<const float4 *>(slot + rd0 + jj * 256);
+                            v[jj] = make_float2(w.x, w.y);
+                            v[jj + 1] = make_float2(w.z, w.w);
+                        }
+                    } else {
+#pragma unroll
+                        for (int jj = 0; jj < 16; ++jj)
+                            v[jj] = *reinterpret_cast<const float2 *>(slot + ((jj & 1) ? rd1 : rd0) + (jj / 2) * 512);
+                    }
+                    put16(abase, acol_in(h, ch), v);
+                }
+                if (!ok) break;
+                asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(bar_full_h(b, h));
+            }
         }
         asm volatile("cp.async.wait_all;" ::: "memory");
     } else if (warp < kLoaderWarps) {
@@ -441,33 +644,71 @@ __global__ void __launch_bounds__(tc::kThreads, 1) k_fused_tc(const __grid_const
         const int q = e & 3, h = e >> 2;
         const int srow = 32 * q + lane;
         // Lowest target on index bit 0: the thread writes amplitudes j and j+1 of its slice
-        // (adjacent) as one 16-byte store. On bit 1: index bit 0 is the lowest slice bit, and
+        // (adjacent) as one 16-byte store, or with the next one on bit 1 four of them as one of
+        // 32 bytes. On bits 1..4: index bit 0 is the lowest slice bit, and
         // lane pairs swap one amplitude so that each lane writes two adjacent slices of one j
         // (the even lane j, the odd lane j+1). Either way a store instruction covers 512
-        // contiguous bytes; otherwise 8-byte stores already fill whole 32-byte sectors.
-        const int smode = t[0] == 0 ? 1 : (t[0] == 1 ? 2 : 0);
+        // contiguous bytes (with one target below bit 6); above bit 4, 8-byte stores already
+        // fill whole lines.
+        const int smode = t[0] == 0 ? (t[1] == 1 ? 3 : 1) : (t[0] < 5 ? 2 : 0);
         const bool odd = lane & 1;
-        auto st16 = [](float2 *p, float2 x, float2 y) {
-            asm volatile("st.global.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(p), "f"(x.x), "f"(x.y), "f"(y.x), "f"(y.y)
-                         : "memory");
+        // on bits 1..4 the lane's row is the even slice of its pair, and odd lanes start at j + 1
+        const uint64_t ebase = row_bytes(smode == 2 ? srow & ~1 : srow) + (h ? ps.joff5 : 0ull) +
+                               (smode == 2 && odd ? ps.joff[1] : 0ull);
+        // Chain: what the last pass stores is not read again, so it leaves L2 first, and the chunks
+        // that wait for their next pass stay (without it a window of 96 MB overflows L2: 281 against
+        // 248 us a pass at 27 qubits).
+        uint64_t policy = 0;
+        if constexpr (kChain) {
+            if (pidx + 1 == uint32_t(a.npass))
+                asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(policy));
+            else
+                asm volatile("createpolicy.fractional.L2::evict_normal.b64 %0, 1.0;" : "=l"(policy));
+        }
+        auto st16 = [policy](uint8_t *p, float2 x, float2 y) {
+            if constexpr (kChain)
+                asm volatile("st.global.L2::cache_hint.v4.f32 [%0], {%1, %2, %3, %4}, %5;" ::"l"(p), "f"(x.x), "f"(x.y),
+                             "f"(y.x), "f"(y.y), "l"(policy)
+                             : "memory");
+            else
+                asm volatile("st.global.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(p), "f"(x.x), "f"(x.y), "f"(y.x), "f"(y.y)
+                             : "memory");
+        };
+        auto st32 = [policy](uint8_t *p, float2 x, float2 y, float2 z, float2 w) {
+            if constexpr (kChain)
+                asm volatile("st.global.L2::cache_hint.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8}, %9;" ::"l"(p),
+                             "f"(x.x), "f"(x.y), "f"(y.x), "f"(y.y), "f"(z.x), "f"(z.y), "f"(w.x), "f"(w.y), "l"(policy)
+                             : "memory");
+            else
+                asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "f"(x.x), "f"(x.y),
+                             "f"(y.x), "f"(y.y), "f"(z.x), "f"(z.y), "f"(w.x), "f"(w.y)
+                             : "memory");
+        };
+        auto st8 = [policy](uint8_t *p, float2 x) {
+            if constexpr (kChain)
+                asm volatile("st.global.L2::cache_hint.v2.f32 [%0], {%1, %2}, %3;" ::"l"(p), "f"(x.x), "f"(x.y), "l"(policy)
+                             : "memory");
+            else
+                *reinterpret_cast<float2 *>(p) = x;
         };
         for (uint32_t i = 0; i < my_tiles; ++i) {
             const int b = i & 1;
             if (!warp_wait<!kTf32>(bar_done(b), (i >> 1) & 1, abort_flag, lim)) break;
             tc_fence_after();
-            const uint64_t tile = uint64_t(blockIdx.x) + uint64_t(i) * gridDim.x;
-            const uint64_t base = slice_base(tile * M + srow, t);
+            uint8_t *dst = reinterpret_cast<uint8_t *>(a.psi) + (ebase | tile_bytes((cta + i * ctas) ^ a.flip));
             const uint32_t dbase = dcol_of(b) + (uint32_t(32 * q) << 16);
 #pragma unroll
             for (int c = 0; c < 2; ++c) {
                 float2 v[16];
                 get16(dbase, 32 * h + 16 * c, v);
-                const int j0 = 32 * h + 16 * c;
-                if (smode == 1) {
+                if (smode == 3) {
 #pragma unroll
-                    for (int jj = 0; jj < 16; jj += 2) st16(a.psi + (base | off[j0 + jj]), v[jj], v[jj + 1]);
+                    for (int jj = 0; jj < 16; jj += 4)
+                        st32(dst + ps.joff[16 * c + jj], v[jj], v[jj + 1], v[jj + 2], v[jj + 3]);
+                } else if (smode == 1) {
+#pragma unroll
+                    for (int jj = 0; jj < 16; jj += 2) st16(dst + ps.joff[16 * c + jj], v[jj], v[jj + 1]);
                 } else if (smode == 2) {
-                    const uint64_t pbase = base & ~1ull;  // the even slice of the lane pair
 #pragma unroll
                     for (int jj = 0; jj < 16; jj += 2) {
                         // selects, not branches: one 16-byte store instruction for the whole warp
@@ -475,16 +716,23 @@ __global__ void __launch_bounds__(tc::kThreads, 1) k_fused_tc(const __grid_const
                         const float2 recv = make_float2(__shfl_xor_sync(0xffffffffu, send.x, 1),
                                                         __shfl_xor_sync(0xffffffffu, send.y, 1));
                         const float2 x = odd ? recv : v[jj], y = odd ? v[jj + 1] : recv;
-                        st16(a.psi + (pbase | off[j0 + jj + (odd ? 1 : 0)]), x, y);
+                        st16(dst + ps.joff[16 * c + jj], x, y);
                     }
                 } else {
 #pragma unroll
-                    for (int jj = 0; jj < 16; ++jj) a.psi[base | off[j0 + jj]] = v[jj];
+                    for (int jj = 0; jj < 16; ++jj) st8(dst + ps.joff[16 * c + jj], v[jj]);
                 }
             }
             tc_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive(bar_free(b));
+            if constexpr (kChain) {
+                const uint32_t c = (cta + i * ctas) >> a.clog;
+                if (lane == 0 && (i + 1 == my_tiles || ((cta + (i + 1) * ctas) >> a.clog) != c)) {
+                    __threadfence_block();  // this warp's stores (ordered by the warp barrier) before the count
+                    chunk_out[e] = c + 1;
+                }
+            }
         }
     } else if (warp < kLoaderWarps + kEpiWarps) {
         // ---------------------------------------------------------------- epilogue (memory order)
@@ -522,6 +770,71 @@ __global__ void __launch_bounds__(tc::kThreads, 1) k_fused_tc(const __grid_const
             __syncwarp();
             if (lane == 0) mbar_arrive(bar_sfree(b));
         }
+    } else if (kChain && warp == kLoaderWarps + kEpiWarps + 1) {
+        // ---------------------------------------------------------------- chain: which chunks may start
+        if (lane == 0 && my_tiles > 0) {
+            const uint32_t chunks = ntile >> a.clog;
+            const uint32_t need = ((cta + (my_tiles - 1) * ctas) >> a.clog) + 1;
+            const uint32_t whole = 1u << a.clog;
+            const uint32_t *in = a.sync + 1 + (pidx - 1) * chunks;   // the pass before (pidx > 0)
+            const uint32_t *out = a.sync + 1 + (pidx + 1) * chunks;  // the pass after (pidx < npass - 1)
+            uint32_t avail = pidx == 0 ? chunks : 0u, taken = 0, told = 0;
+            const bool last = pidx + 1 == uint32_t(a.npass);
+            auto ld = [](const uint32_t *q) {
+                uint32_t v;
+                asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(q) : "memory");
+                return v;
+            };
+            long long t0 = clock64();
+            while (told < need && !*abort_flag) {
+                while (avail < chunks && ld(in + avail) >= whole) ++avail;
+                while (!last && taken < chunks && taken + a.window < need && ld(out + taken) >= whole) ++taken;
+                const uint32_t now = last ? avail : min(avail, taken + a.window);
+                if (now > told) {
+                    told = now;
+                    __threadfence_block();
+                    *chunk_limit = told;
+                    t0 = clock64();
+                } else if (*reinterpret_cast<volatile uint32_t *>(a.sync)) {
+                    *abort_flag = 1;
+                } else if (clock64() - t0 > lim) {
+                    *abort_flag = 1;
+                } else {
+                    __nanosleep(100);
+                }
+            }
+        }
+        __syncwarp();
+    } else if (kChain && warp == kLoaderWarps + kEpiWarps + 2) {
+        // ---------------------------------------------------------------- chain: publish stored chunks
+        const uint32_t chunks = ntile >> a.clog;
+        for (uint32_t i = 0; i < my_tiles;) {
+            const uint32_t c = (cta + i * ctas) >> a.clog;
+            uint32_t n = 1;  // the CTA's tiles of chunk c
+            while (i + n < my_tiles && ((cta + (i + n) * ctas) >> a.clog) == c) ++n;
+            const long long t0 = clock64();
+            bool stop = false;
+            for (;;) {
+                const bool out = lane >= kEpiWarps || chunk_out[lane] > c;
+                if (__all_sync(0xffffffffu, out)) break;
+                int s = 0;
+                if (lane == 0) {
+                    if (*abort_flag) s = 1;
+                    else if (clock64() - t0 > lim) *abort_flag = s = 1;
+                }
+                if ((stop = __shfl_sync(0xffffffffu, s, 0) != 0)) break;
+                __nanosleep(100);
+            }
+            if (stop) break;
+            __threadfence_block();
+            __syncwarp();
+            if (lane == 0) {
+                __threadfence();  // release: the epilogue warps' stores, seen above, before the count
+                atomicAdd(a.sync + 1 + pidx * chunks + c, n);
+            }
+            i += n;
+        }
+        __syncwarp();
     } else {
         // ---------------------------------------------------------------- MMA issuer
         if (lane == 0) {
@@ -598,7 +911,10 @@ __global__ void __launch_bounds__(tc::kThreads, 1) k_fused_tc(const __grid_const
 
     tc_fence_before();
     __syncthreads();
-    if (threadIdx.x == 0 && *abort_flag) atomicOr(a.err, 8);
+    if (threadIdx.x == 0 && *abort_flag) {
+        atomicOr(a.err, kErrTimeout);
+        if constexpr (kChain) atomicExch(a.sync, 1u);
+    }
     if (warp == kLoaderWarps + kEpiWarps) {
         tc_fence_after();
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTmemCols) : "memory");
@@ -713,9 +1029,9 @@ void tc_build_ops(const Pass &p, void *host_image, bool tf32) {
     else build_ops_bf16(p, img);
 }
 
-template <bool kStaged, bool kTf32, bool kSub = false>
+template <bool kStaged, bool kTf32, bool kSub = false, bool kChain = false>
 static int set_smem_attr() {
-    const cudaError_t e = cudaFuncSetAttribute(k_fused_tc<kStaged, kTf32, kSub>,
+    const cudaError_t e = cudaFuncSetAttribute(k_fused_tc<kStaged, kTf32, kSub, kChain>,
                                                cudaFuncAttributeMaxDynamicSharedMemorySize, tc::Layout<kTf32>::kAlloc);
     return e == cudaSuccess ? RCS_OK : note_launch_error("tensor-core kernel shared-memory attribute", e);
 }
@@ -731,32 +1047,80 @@ int tc_prepare_device() {
     if (rc == RCS_OK) rc = set_smem_attr<true, true>();
     if (rc == RCS_OK) rc = set_smem_attr<false, false, true>();
     if (rc == RCS_OK) rc = set_smem_attr<false, true, true>();
+    if (rc == RCS_OK) rc = set_smem_attr<false, false, false, true>();
     if (rc == RCS_OK && dev >= 0 && dev < 64) attr_done[dev] = true;
     return rc;
 }
 
-static int launch_tc(void *psi, int n, const Pass &p, const void *d_ops, int *d_err, void *stream, bool tf32,
-                     const void *sub, uint64_t tmask) {
-    using namespace tc;
-    if (p.k != K || n < K + 7) return RCS_ERR_UNSUPPORTED;
-    if (int rc = tc_prepare_device(); rc != RCS_OK) return rc;
-    TcArgs a;
-    a.psi = static_cast<float2 *>(psi);
-    a.sub = static_cast<const float2 *>(sub);
-    a.tmask = tmask;
-    a.ops = static_cast<const uint4 *>(d_ops);
-    a.err = d_err;
-    tc_test_fault(&a.wait_cycles, &a.skip_tile);
-    a.tiles = uint32_t((1ull << (n - K)) / M);
-    for (int i = 0; i < K; ++i) a.t[i] = p.t[i];
-    // qubits varying inside a tile: the targets plus the 7 lowest other qubits
+// The qubits that vary inside a tile of pass p: its targets and the 7 lowest other qubits.
+static uint64_t tile_qubits(const Pass &p, int n) {
     uint64_t V = 0;
-    for (int i = 0; i < K; ++i) V |= 1ull << p.t[i];
+    for (int i = 0; i < tc::K; ++i) V |= 1ull << p.t[i];
     for (int qb = 0, k = 0; qb < n && k < 7; ++qb)
-        if (!((V >> qb) & 1) && !(std::find(p.t, p.t + K, qb) != p.t + K)) {
+        if (!((V >> qb) & 1)) {
             V |= 1ull << qb;
             ++k;
         }
+    return V;
+}
+
+// Kernel form of pass p on n qubits. `chunk` holds the qubits of a chunk (a superset of the
+// tile's): the tile number counts through them first, then through the others.
+static void fill_pass(const Pass &p, int n, const void *d_ops, uint64_t chunk, TcPass *out) {
+    using namespace tc;
+    out->ops = static_cast<const uint4 *>(d_ops);
+    for (int i = 0; i < K; ++i) out->t[i] = p.t[i];
+    for (int j = 0; j < 32; ++j) {
+        out->joff[j] = 0;
+        for (int i = 0; i < 5; ++i)
+            if ((j >> i) & 1) out->joff[j] |= 8ull << p.t[i];
+    }
+    out->joff5 = 8ull << p.t[5];
+    const bool quad = p.t[0] == 0 && p.t[1] == 1;  // see the slice-order loader
+    const uint64_t V = tile_qubits(p, n);
+    std::fill(out->tpos, out->tpos + 32, int8_t(-1));
+    int r = 0, tb = 0;
+    for (int qb = 0; qb < n; ++qb)
+        if (((V >> qb) & 1) && std::find(p.t, p.t + K, qb) == p.t + K) out->rpos[r++] = int8_t(qb);
+    for (int c = 0; c < 8; ++c)
+        out->coff[c] = quad ? ((c & 1) ? 8ull << out->rpos[4] : 0ull) + out->joff[4 * (c >> 1)] : out->joff[2 * c];
+    for (int inside = 1; inside >= 0; --inside)
+        for (int qb = 0; qb < n; ++qb)
+            if (!((V >> qb) & 1) && int((chunk >> qb) & 1) == inside) out->tpos[tb++] = int8_t(qb);
+}
+
+static int low_targets(const Pass &p) {
+    int low = 0;
+    for (int i = 0; i < tc::K; ++i) low += p.t[i] < 5;
+    return low;
+}
+
+static int launch_tc(void *psi, int n, const Pass &p, const void *d_ops, int *d_err, void *stream, bool tf32,
+                     const void *sub, uint64_t tmask, bool backwards) {
+    using namespace tc;
+    if (p.k != K || n < K + 7) return RCS_ERR_UNSUPPORTED;
+    if (int rc = tc_prepare_device(); rc != RCS_OK) return rc;
+    TcArgs<1> a;
+    a.psi = static_cast<float2 *>(psi);
+    a.sub = static_cast<const float2 *>(sub);
+    a.tmask = tmask;
+    a.err = d_err;
+    tc_test_fault(&a.wait_cycles, &a.skip_tile);
+    a.npass = 1;
+    a.clog = 0;
+    a.window = 0;
+    a.sync = nullptr;
+    a.tiles = uint32_t((1ull << (n - K)) / M);
+    // the memory-order and sub-state loaders walk forwards
+    const bool staged = low_targets(p) >= 4;
+    a.flip = backwards && !staged && !sub ? a.tiles - 1 : 0;
+    // A state beyond L2 streams best with one tile (two units) in flight per SM: with all five
+    // units HBM serves the same bytes more slowly (328 against 351 us a BF16x3 pass at 27 qubits;
+    // from L2 five units are faster, 23.4 against 24.7 us at 23). TF32x3 times alike with 2 to 4.
+    a.depth = !tf32 && (8ull << n) > (uint64_t(64) << 20) ? 2u : uint32_t(tf32 ? Layout<true>::kSlots : Layout<false>::kSlots);
+    // qubits varying inside a tile: the targets plus the 7 lowest other qubits
+    const uint64_t V = tile_qubits(p, n);
+    fill_pass(p, n, d_ops, V, &a.pass[0]);
     a.vmask = V;
     a.r = 0;
     while (a.r < 64 && ((V >> a.r) & 1)) ++a.r;
@@ -765,38 +1129,113 @@ static int launch_tc(void *psi, int n, const Pass &p, const void *d_ops, int *d_
     // slice-order variant streams at full rate. With 4 or more targets below qubit 5 every slice is
     // a short contiguous run and the memory-order variant is faster (158 -> 79 ms for targets 0..5
     // at 34 qubits); for fewer low targets the slice-order variant measured faster.
-    int low = 0;
-    for (int i = 0; i < K; ++i) low += p.t[i] < 5;
-    const bool staged = low >= 4;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     if (sub) {
         if (staged) return RCS_ERR_UNSUPPORTED;  // the sub-state input has a slice-order loader only
-        if (tf32) k_fused_tc<false, true, true><<<grid, kThreads, Layout<true>::kAlloc, st>>>(a);
-        else k_fused_tc<false, false, true><<<grid, kThreads, Layout<false>::kAlloc, st>>>(a);
+        if (tf32) k_fused_tc<false, true, true, false><<<grid, kThreads, Layout<true>::kAlloc, st>>>(a);
+        else k_fused_tc<false, false, true, false><<<grid, kThreads, Layout<false>::kAlloc, st>>>(a);
     } else if (tf32) {
-        if (staged) k_fused_tc<true, true, false><<<grid, kThreads, Layout<true>::kAlloc, st>>>(a);
-        else k_fused_tc<false, true, false><<<grid, kThreads, Layout<true>::kAlloc, st>>>(a);
+        if (staged) k_fused_tc<true, true, false, false><<<grid, kThreads, Layout<true>::kAlloc, st>>>(a);
+        else k_fused_tc<false, true, false, false><<<grid, kThreads, Layout<true>::kAlloc, st>>>(a);
     } else {
-        if (staged) k_fused_tc<true, false, false><<<grid, kThreads, Layout<false>::kAlloc, st>>>(a);
-        else k_fused_tc<false, false, false><<<grid, kThreads, Layout<false>::kAlloc, st>>>(a);
+        if (staged) k_fused_tc<true, false, false, false><<<grid, kThreads, Layout<false>::kAlloc, st>>>(a);
+        else k_fused_tc<false, false, false, false><<<grid, kThreads, Layout<false>::kAlloc, st>>>(a);
     }
     return launch_status("tensor-core pass");
 }
 
-int launch_pass_tc(void *psi, int n, const Pass &p, const void *d_ops, int *d_err, void *stream, bool tf32) {
-    return launch_tc(psi, n, p, d_ops, d_err, stream, tf32, nullptr, 0);
+int launch_pass_tc(void *psi, int n, const Pass &p, const void *d_ops, int *d_err, void *stream, bool tf32,
+                   bool backwards) {
+    return launch_tc(psi, n, p, d_ops, d_err, stream, tf32, nullptr, 0, backwards);
 }
 
 bool tc_pass_takes_substate(const Pass &p, int n) {
-    int low = 0;
-    for (int i = 0; i < tc::K; ++i) low += p.t[i] < 5;
-    return p.kind == PASS_TC && p.k == tc::K && n >= tc::K + 7 && low < 4;
+    return p.kind == PASS_TC && p.k == tc::K && n >= tc::K + 7 && low_targets(p) < 4;
 }
 
 int launch_pass_tc_from_sub(void *psi, int n, const Pass &p, const void *d_ops, int *d_err, void *stream, bool tf32,
                             const void *sub, uint64_t tmask) {
     if (!sub) return RCS_ERR_ARG;
-    return launch_tc(psi, n, p, d_ops, d_err, stream, tf32, sub, tmask);
+    return launch_tc(psi, n, p, d_ops, d_err, stream, tf32, sub, tmask, false);
+}
+
+// ---------------------------------------------------------------- chains of passes
+
+// The chunk of a chain of `count` passes: every tile's qubits of every pass, filled up with
+// the lowest other qubits to at least kChunkMinLog2. 0 if the passes cannot form a chain.
+static uint64_t chain_chunk(const Pass *const *p, int count, int n) {
+    uint64_t C = 0;
+    for (int i = 0; i < count; ++i) {
+        if (p[i]->kind != PASS_TC || p[i]->k != tc::K || low_targets(*p[i]) >= 4) return 0;
+        C |= tile_qubits(*p[i], n);
+    }
+    for (int qb = 0; qb < n && std::popcount(C) < tc::kChunkMinLog2; ++qb) C |= 1ull << qb;
+    return C;
+}
+
+size_t tc_chain_sync_bytes(int n) {
+    return n < tc::kChainMinQubits ? 0 : (1 + (size_t(tc::kChainMax) << (n - tc::kChunkMinLog2))) * sizeof(uint32_t);
+}
+
+std::vector<int> tc_chain_lengths(const std::vector<Pass> &passes, int n, bool tf32) {
+    const size_t m = passes.size();
+    std::vector<int> len(m, 1);
+    if (n < tc::kChainMinQubits || tf32) return len;
+    // cheapest split of the sequence, from the back
+    std::vector<double> best(m + 1, 0.0);
+    for (size_t i = m; i-- > 0;) {
+        best[i] = 1e300;
+        const Pass *p[tc::kChainMax];
+        for (int c = 1; c <= tc::kChainMax && i + size_t(c) <= m; ++c) {
+            p[c - 1] = &passes[i + size_t(c) - 1];
+            const uint64_t C = chain_chunk(p, c, n);
+            if (c > 1 && (C == 0 || std::popcount(C) > tc::kChunkMaxLog2[c])) break;
+            const double cost = tc::kChainCost[c] + best[i + size_t(c)];
+            if (cost < best[i]) {
+                best[i] = cost;
+                len[i] = c;
+            }
+        }
+    }
+    return len;
+}
+
+int launch_chain_tc(void *psi, int n, const Pass *const *p, const void *const *d_ops, int count, uint32_t *sync,
+                    int *d_err, void *stream, bool backwards) {
+    using namespace tc;
+    if (count < 2 || count > kChainMax || n < kChainMinQubits || !sync) return RCS_ERR_ARG;
+    const uint64_t C = chain_chunk(p, count, n);
+    if (C == 0) return RCS_ERR_ARG;
+    if (int rc = tc_prepare_device(); rc != RCS_OK) return rc;
+    TcArgs<kChainMax> a;
+    std::memset(&a, 0, sizeof(a));
+    a.psi = static_cast<float2 *>(psi);
+    a.err = d_err;
+    tc_test_fault(&a.wait_cycles, &a.skip_tile);
+    a.tiles = uint32_t((1ull << (n - K)) / M);
+    a.npass = count;
+    a.clog = std::popcount(C) - K - 7;
+    a.window = uint32_t(kChainWindowBytes[count] >> (std::popcount(C) + 3));
+    a.sync = sync;
+    a.flip = backwards ? a.tiles - 1 : 0;
+    a.depth = uint32_t(Layout<false>::kSlots);
+    for (int i = 0; i < count; ++i) fill_pass(*p[i], n, d_ops[i], C, &a.pass[i]);
+    cudaStream_t st = static_cast<cudaStream_t>(stream);
+    const size_t words = 1 + size_t(count) * (a.tiles >> a.clog);
+    if (cudaError_t e = cudaMemsetAsync(sync, 0, words * sizeof(uint32_t), st); e != cudaSuccess)
+        return note_launch_error("chain counters", e);
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(unsigned(std::min<uint64_t>(uint64_t(a.tiles) * unsigned(count), uint64_t(device_sm_count()))));
+    cfg.blockDim = dim3(kChainThreads);
+    cfg.dynamicSmemBytes = Layout<false>::kAlloc;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeCooperative;  // the CTAs wait for one another
+    attr[0].val.cooperative = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, k_fused_tc<false, false, false, true>, a);
+    return e == cudaSuccess ? RCS_OK : note_launch_error("chained tensor-core passes", e);
 }
 
 }  // namespace rcs

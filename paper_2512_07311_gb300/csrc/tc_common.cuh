@@ -21,6 +21,25 @@ constexpr int M = 128;          // slices per tile (GEMM M, TMEM lanes)
 constexpr int kLoaderWarps = 8;
 constexpr int kEpiWarps = 8;
 constexpr int kThreads = (kLoaderWarps + kEpiWarps + 1) * 32;  // 544
+// Chains of passes (k_tc.cu).
+constexpr int kChainMax = 3;                    // passes of a chain
+constexpr int kChainThreads = kThreads + 64;    // two more warps order the chunks
+// From 128 MB a state no longer stays in L2 from one pass to the next (two passes at 24 qubits:
+// 87 us as a chain, 95 one after the other; at 23 qubits 57 against 47).
+constexpr int kChainMinQubits = 24;
+// A chunk of 4 MB keeps the CTAs of a pass busy for about one tile each. The larger it is, the
+// fewer of them fit the window below; two passes need chunks of up to 2^19 amplitudes, three
+// mostly 2^19 to 2^21.
+constexpr int kChunkMinLog2 = 19;
+constexpr int kChunkMaxLog2[kChainMax + 1] = {0, 0, 21, 20};
+// Distance between two passes of a chain. The tiles in flight in both (about 4 per SM each) and
+// the counters' round trip take some 70 MB; beyond about 80 MB for a pair and 64 MB a step for
+// three the chunks start to fall out of L2. Measured at 27 qubits, us a pass: pairs with 40 /
+// 56 / 72 / 80 / 96 / 128 MB 301 / 259 / 233 / 229 / 248 / 288; threes with 20 / 32 / 48 / 64 MB
+// 416 / 289 / 243 / 230.
+constexpr uint64_t kChainWindowBytes[kChainMax + 1] = {0, 0, uint64_t(80) << 20, uint64_t(64) << 20};
+// Time of a chain in passes of one launch each (350 us before, 229 a pass in pairs and threes).
+constexpr double kChainCost[kChainMax + 1] = {0, 1.0, 1.36, 2.06};
 constexpr int kOpBytes = NR * KR * 2;                          // one bf16 operand image: 32 KB
 constexpr int kStageBytes = D * M * 8;                         // one tile of complex64: 64 KB
 constexpr int kSmBhi = 0;                                      // BF16: B_hi image, then B_lo
@@ -30,20 +49,23 @@ constexpr int kSmBlo = kOpBytes;
 constexpr int kTf32Rows = 3 * D;
 constexpr int kTf32Atom = kTf32Rows * 128;   // 24 KB
 constexpr int kTf32Split = 2 * kTf32Atom;    // 48 KB
-// Shared-memory map (offsets from a 1024-aligned base): the B images, two stages of
-// one tile each, then the small tables.
+constexpr int kSlotBytes = 4096;  // slice-order loaders: one unit of 16 amplitudes x 32 slices
+// Shared-memory map (offsets from a 1024-aligned base): the B images, the stage (two of
+// one tile each, or kSlots units per loader warp), then the small tables.
 template <bool kTf32>
 struct Layout {
     static constexpr int kBBytes = kTf32 ? 2 * kTf32Split : 2 * kOpBytes;
     static constexpr int kStage0 = kBBytes;
-    static constexpr int kOff = kStage0 + 2 * kStageBytes;  // 64 x u64 target offsets
+    static constexpr int kSlots = kTf32 ? 4 : 5;  // what fits beside the B images
+    static constexpr int kOff = kStage0 + kLoaderWarps * kSlots * kSlotBytes;  // 64 x u64 target offsets
     static constexpr int kHiOff = kOff + D * 8;             // 64 x u64 offsets of the high compact bits
     static constexpr int kCj = kHiOff + 64 * 8;             // 64 x u16 compact index of local amplitude j
     static constexpr int kCs = kCj + D * 2;                 // 128 x u16 compact index of slice s within the tile
     static constexpr int kBar = kCs + M * 2;                // 16 mbarriers
-    static constexpr int kMisc = kBar + 16 * 8;             // tmem slot, abort flag
-    static constexpr int kAlloc = kMisc + 16 + 1024;        // slack for 1024-byte alignment
+    static constexpr int kMisc = kBar + 16 * 8;             // tmem slot, abort flag, chain: chunk limit, 8 counts
+    static constexpr int kAlloc = kMisc + 48 + 1024;        // slack for 1024-byte alignment
     static_assert(kAlloc <= 227 * 1024, "shared memory");
+    static_assert(kLoaderWarps * kSlots * kSlotBytes >= 2 * kStageBytes, "the stage of the other variants");
 };
 constexpr uint32_t kTmemCols = 512;
 // instruction descriptor: D f32, A bf16, B bf16, both K-major, N = 128, M = 128

@@ -307,36 +307,14 @@ BitMap to_stored(const rcs_ctx *c) {
     return m;
 }
 
-// Brings the stored state back to the identity layout with exact swap passes
-// (entries 0 and 1, so FP32 moves the amplitudes unchanged).
+// Brings the stored state back to the identity layout (the amplitudes move unchanged).
 int restore_layout(rcs_ctx *c) {
-    if (c->zero_pending) {  // |0...0> in any layout
-        set_identity_layout(c);
-        return RCS_OK;
+    if (!c->zero_pending) {  // |0...0> is the same in any layout
+        if (launch_restore_layout(c->psi, c->n, c->phys_of, c->stream) != RCS_OK)
+            return fail(c, RCS_ERR_CUDA, "layout change: " + take_launch_error());
+        c->sums_valid = false;
     }
-    int log_of[64];
-    for (int q = 0; q < c->n; ++q) log_of[c->phys_of[q]] = q;
-    for (int p = 0; p < c->n; ++p) {
-        while (log_of[p] != p) {
-            const int l = log_of[p];
-            const int q = c->phys_of[p];  // where circuit qubit p sits now
-            Pass sw;
-            sw.kind = PASS_2Q;
-            sw.k = 2;
-            for (int i = 0; i < 8; ++i) sw.t[i] = -1;
-            sw.t[0] = std::min(p, q);
-            sw.t[1] = std::max(p, q);
-            sw.U.assign(16, cd(0.0));
-            sw.U[0] = sw.U[6] = sw.U[9] = sw.U[15] = 1.0;
-            if (launch_pass_plain(c->psi, c->n, sw, c->stream) != RCS_OK)
-                return fail(c, RCS_ERR_CUDA, "layout swap: " + take_launch_error());
-            c->phys_of[p] = p;
-            c->phys_of[l] = q;
-            log_of[p] = p;
-            log_of[q] = l;
-        }
-    }
-    c->sums_valid = false;
+    set_identity_layout(c);
     return RCS_OK;
 }
 

@@ -1005,11 +1005,29 @@ int rcs_batch_state_read(rcs_batch *b, size_t i, uint64_t first, uint64_t count,
         BCUDA(b, cudaMemcpy(out_re_im, h.psi + first, count * 8, cudaMemcpyDeviceToHost), "read state");
         return RCS_OK;
     }
-    // stored in the plan's qubit layout: read it all and put caller index c at position c
+    // stored in the plan's qubit layout: a kernel puts pieces of up to 64 MB into the caller's
+    // order (2^16 amplitudes rearranged on the host took 1 ms; the copy takes 0.05)
+    const BitMap m = plan_to_stored(h.plan);
+    const uint64_t piece = std::min<uint64_t>(count, uint64_t(1) << 23);
+    void *scratch = nullptr;
+    if (cudaMalloc(&scratch, piece * 8) == cudaSuccess) {
+        int rc = RCS_OK;
+        cudaError_t e = cudaSuccess;
+        for (uint64_t off = 0; off < count && rc == RCS_OK && e == cudaSuccess; off += piece) {
+            const uint64_t len = std::min(piece, count - off);
+            rc = launch_read_mapped(h.psi, first + off, len, m, scratch, nullptr);
+            if (rc == RCS_OK) e = cudaMemcpy(out_re_im + 2 * off, scratch, len * 8, cudaMemcpyDeviceToHost);
+        }
+        cudaFree(scratch);
+        if (rc != RCS_OK) return bfail(b, rc, "read state: " + take_launch_error());
+        BCUDA(b, e, "read state");
+        return RCS_OK;
+    }
+    cudaGetLastError();
+    // no device memory left: read it all and rearrange it on the host
     try {
         std::vector<float2> all(static_cast<size_t>(lim));
         BCUDA(b, cudaMemcpy(all.data(), h.psi, lim * 8, cudaMemcpyDeviceToHost), "read state");
-        const BitMap m = plan_to_stored(h.plan);
         float2 *out = reinterpret_cast<float2 *>(out_re_im);
         for (uint64_t c = first; c < first + count; ++c) {
             uint64_t s = 0;

@@ -460,7 +460,7 @@ int launch_plan_pass(void *psi, int n, const Pass &p, const uint8_t *ops, int *d
     switch (p.kind) {
         case PASS_1Q:
         case PASS_2Q: return launch_pass_plain(psi, n, p, stream);
-        case PASS_SIMT: return launch_pass_simt(psi, n, p, ops, stream);
+        case PASS_SIMT: return launch_pass_simt(psi, n, p, ops, stream, backwards);
         case PASS_TC: return launch_pass_tc(psi, n, p, ops, d_err, stream, tf32, backwards);
         default: return RCS_ERR_ARG;
     }

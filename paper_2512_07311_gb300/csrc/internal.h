@@ -153,7 +153,8 @@ int launch_pass_plain(void *psi, int n, const Pass &p, void *stream);
 // Fused FP32 SIMT pass of width p.k = 1..kSimtKMax. Widths up to kSimtParamK carry U in
 // the kernel parameters (ops unused); wider ones read it from ops, the device copy of
 // simt_build_ops(p) (16-byte aligned), and give RCS_ERR_ARG without it.
-int launch_pass_simt(void *psi, int n, const Pass &p, const uint8_t *ops, void *stream);
+// backwards as for launch_pass_tc (widths up to kSimtParamK).
+int launch_pass_simt(void *psi, int n, const Pass &p, const uint8_t *ops, void *stream, bool backwards = false);
 // Bytes of a SIMT pass's device image (0 for widths up to kSimtParamK) and its builder.
 size_t simt_ops_bytes(int k);
 void simt_build_ops(const Pass &p, uint8_t *out);

@@ -8,14 +8,17 @@
 //    flop per byte, far below the FP32 ridge.
 //  * k_fused_simt<K>: one launch per fused K-qubit unitary (K <= 4). Thread =
 //    one slice of 2^K amplitudes (the amplitudes that differ only in the target
-//    bits); lanes of a warp take consecutive slices, so each load instruction
-//    covers consecutive addresses along the lowest non-target qubits. The
-//    unitary travels in the kernel's parameter space (constant bank) and the
-//    fully unrolled complex mat-vec reads it as immediate constant operands.
-//    8 * 2^K real flop per amplitude: HBM-bound up to K = 4 on GB300.
+//    bits); lanes of a warp take consecutive slices, so each copy covers
+//    consecutive addresses along the lowest qubits. The unitary travels in the
+//    kernel's parameter space (constant bank) and the fully unrolled complex
+//    mat-vec reads it as constant operands. 8 * 2^K real flop per amplitude:
+//    HBM-bound up to K = 4 on GB300 (at K = 4 just so: the packed multiply-adds
+//    reach 68 TFLOP/s with nothing else to do, 253 us of a pass of 340).
 //  * k_fused_wide<K>: fused K = 5, 6 or 7 qubit unitaries, a CTA per tile of 128
 //    (K = 5) or 64 slices, U from a device image in shared memory (see below).
 //    Bound by the FP32 FMA pipe.
+#include <algorithm>
+
 #include "dev_common.cuh"
 #include "internal.h"
 
@@ -148,89 +151,205 @@ struct CEnt {
     float2 rr, ni;
 };
 
+// Slice-order addressing, in bytes: a unit's base | a lane's base | a local amplitude's
+// offset. The offsets and U are constant operands.
 template <int K>
 struct SimtArgs {
     CEnt U[1 << K][1 << K];
-    int t[K];  // ascending
-    uint64_t slices;
+    uint64_t joff[1 << K];        // local amplitude j
+    uint64_t coff[1 << (K - 1)];  // copy c of a unit (see k_fused_simt)
+    uint64_t units;
+    uint32_t depth;               // units in a warp's ring, 2..kSimtSlots
+    uint32_t flip;                // XORed into the unit numbers: 0, or units - 1 to walk the state backwards
+    int t[K];                     // ascending
+    int8_t rpos[5];               // index bit of lane (slice) bit i: the 5 lowest non-target qubits
+    int8_t upos[32];              // index bit of unit number bit i: the other qubits (-1: none)
 };
 
-// Resident CTAs per SM for width K, set by the registers the mat-vec needs without
-// spilling (the two stages of 256 slices x 2^K amplitudes fit in shared memory).
+// CTAs of 8 warps per SM. At width 1 a unit is 512 bytes, and two CTAs do not keep enough in
+// flight (371 against 326 us at 27 qubits); at width 4 three slow HBM down (340 against 370).
 template <int K>
 constexpr int simt_blocks_per_sm() {
-    return K == 4 ? 2 : 3;
+    return K == 1 ? 3 : 2;
+}
+template <int K>
+constexpr uint32_t simt_unit_bytes() {
+    return 256u << K;  // 32 slices of 2^K amplitudes
+}
+constexpr uint32_t kSimtSlots = 3;  // of a warp's ring
+// Units a warp keeps in its ring: the one it multiplies and one or two in flight. HBM serves
+// wide copies best with no more in flight than it needs. At 27 qubits, two against three:
+// width 4 with the lowest target on bits 1..4 340 and 350 us, with none below bit 5 360 and 335;
+// width 3 330 and 360; width 2 360 and 326 (one 8-byte copy per amplitude through L1, one slice
+// per thread in flight: 351-361, 342-347, 330-335).
+template <int K>
+uint32_t simt_depth(int lowest) {
+    return K == 3 || (K == 4 && lowest < 5) ? 2u : 3u;
 }
 
-// One thread per 2^K-amplitude slice, persistent over the slices (grid-stride). Each
-// thread double-buffers its own slice through shared memory with cp.async: the copies of
-// its next slice are in flight while it multiplies the current one, so the loads of a
-// slice never wait behind the previous slice's mat-vec and stores. The stage slots are
-// private to the thread (slot [b][j][thread]), so no block barrier is needed; lanes of a
-// warp take neighbouring slices, and with no target below qubit 5 every copy and store
-// instruction of a warp covers 256 contiguous bytes.
+// A warp applies U to a unit of 32 neighbouring slices, one per lane, persistent over the
+// units (grid-stride). Units come through a ring of shared-memory slots of the warp's own, so
+// the copies of the next ones are in flight while it multiplies, and no block barrier is
+// needed. Copies are 16 bytes wide and bypass L1: for each pair of amplitudes (j = 2 c,
+// 2 c + 1, which differ in the lowest target) the unit's 64 values are one 512-byte block in
+// the order of their index bits: bit tb is the lowest target (bit 5 if that lies above bit 4),
+// the others are the lane bits. So the lanes of a copy go up both in memory and in the slot.
+// With tb = 2 or 3 the blocks' lines 1 and 3 have their halves or sectors swapped, which keeps
+// the reads on different banks; with targets on bits 0 and 1 (quad) neighbouring lanes take
+// the two halves of a 32-byte sector, amplitudes 4 i .. 4 i + 3 of one slice. Outputs leave in
+// 16 bytes (32 in quad) while the lowest target is below bit 5: a slice's j, j + 1 where that
+// is bit 0, else lane pairs swap one output and store two slices' j (even lane) or j + 1.
 template <int K>
-__global__ void __launch_bounds__(256, simt_blocks_per_sm<K>()) k_fused_simt(float2 *__restrict__ psi, const SimtArgs<K> a) {
+__global__ void __launch_bounds__(256, simt_blocks_per_sm<K>())
+    k_fused_simt(float2 *__restrict__ psi, const __grid_constant__ SimtArgs<K> a) {
     constexpr int D = 1 << K;
-    extern __shared__ float2 stage[];  // [2][D][256]
-    // target offsets of local index j, warp-uniform; read back through a volatile
-    // pointer at every use so they are not held in registers across the mat-vec
-    __shared__ uint64_t offs_s[D];
-    if (threadIdx.x < D) {
+    constexpr uint32_t kUnit = simt_unit_bytes<K>();
+    extern __shared__ __align__(16) unsigned char simt_smem[];
+    const int lane = threadIdx.x & 31;
+    const uint32_t warps = gridDim.x * 8u;
+    const int tb = a.t[0] < 5 ? a.t[0] : 5;
+    const bool quad = K > 1 && a.t[0] == 0 && a.t[K > 1] == 1;
+    const bool odd = lane & 1;
+    auto row = [&](int r) {
         uint64_t o = 0;
 #pragma unroll
-        for (int i = 0; i < K; ++i)
-            if ((threadIdx.x >> i) & 1) o |= 1ull << a.t[i];
-        offs_s[threadIdx.x] = o;
-    }
-    __syncthreads();
-    const volatile uint64_t *offs = offs_s;
-    const uint64_t stride = uint64_t(gridDim.x) * blockDim.x;
-    const uint32_t slot0 = uint32_t(__cvta_generic_to_shared(stage)) + threadIdx.x * 8u;
-    auto base_of = [&](uint64_t sl) {
-        uint64_t b = sl;
-#pragma unroll
-        for (int i = 0; i < K; ++i) b = insert_zero(b, a.t[i]);
-        return b;
+        for (int i = 0; i < 5; ++i)
+            if ((r >> i) & 1) o |= 8ull << a.rpos[i];
+        return o;
     };
-    auto issue = [&](uint64_t sl, int buf) {
-        if (sl < a.slices) {
-            const float2 *p = psi + base_of(sl);
+    // copies: this lane's first value of a block, and its place in the slot
+    const uint32_t swl = (tb == 2 || tb == 3) ? ((uint32_t(lane) >> 3) & 1u) << (tb - 1) : 0u;
+    const int cs0 = quad ? lane >> 1 : ((2 * lane) & ((1 << tb) - 1)) | (((2 * lane) >> (tb + 1)) << tb);
+    const uint64_t cbase =
+        row(cs0) | (quad ? (odd ? a.joff[K > 1 ? 2 : 0] : 0ull) : (((2 * lane) >> tb) & 1) ? a.joff[1] : 0ull);
+    unsigned char *ring = simt_smem + (threadIdx.x >> 5) * (kSimtSlots * kUnit);
+    const uint32_t cdst = uint32_t(__cvta_generic_to_shared(ring)) + ((uint32_t(lane) ^ swl) << 4);
+    // reads: where this lane's slice sits in a block, j even and j odd (quad: j mod 4 < 2 and >= 2)
+    uint32_t rd0 = ((uint32_t(lane) >> tb) << (tb + 1)) | (uint32_t(lane) & ((1u << tb) - 1u));
+    if (tb == 2 || tb == 3) rd0 ^= ((rd0 >> 4) & 1u) << tb;
+    rd0 *= 8u;
+    uint32_t rd1 = rd0 ^ (8u << tb);
+    if (quad) {
+        rd0 = (uint32_t(lane) & 15u) * 32u + (uint32_t(lane) >> 4) * 512u;
+        rd1 = rd0 + 16u;
+    }
+    // stores
+    const int smode = quad ? 3 : tb == 0 ? 1 : tb < 5 ? 2 : 0;
+    const uint64_t sbase = row(smode == 2 ? lane & ~1 : lane) | (smode == 2 && odd ? a.joff[1] : 0ull);
+    const int up = a.upos[lane];
+    const uint64_t ubit = up >= 0 ? 8ull << up : 0ull;
+    auto unit_base = [&](uint32_t u) {
+        const bool on = ((u ^ a.flip) >> lane) & 1u;
+        const uint32_t lo = __reduce_or_sync(0xffffffffu, on ? uint32_t(ubit) : 0u);
+        const uint32_t hi = __reduce_or_sync(0xffffffffu, on ? uint32_t(ubit >> 32) : 0u);
+        return (uint64_t(hi) << 32) | lo;
+    };
+    auto issue = [&](uint32_t u, uint32_t slot) {
+        if (u < a.units) {
+            const unsigned char *p = reinterpret_cast<const unsigned char *>(psi) + (cbase | unit_base(u));
 #pragma unroll
-            for (int j = 0; j < D; ++j) {
-                const uint32_t dst = slot0 + uint32_t((buf * D + j) * 256) * 8u;
-                asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(dst), "l"(p + offs[j]) : "memory");
-            }
+            for (int c = 0; c < D / 2; ++c)
+                asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(cdst + slot * kUnit + uint32_t(c) * 512u),
+                             "l"(p + a.coff[c])
+                             : "memory");
         }
         asm volatile("cp.async.commit_group;" ::: "memory");
     };
-    uint64_t s = uint64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-    issue(s, 0);
-    int buf = 0;
+    auto st16 = [](unsigned char *p, float2 x, float2 y) {
+        asm volatile("st.global.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(p), "f"(x.x), "f"(x.y), "f"(y.x), "f"(y.y)
+                     : "memory");
+    };
+    uint32_t u = blockIdx.x * 8u + (threadIdx.x >> 5);
+    const bool deep = a.depth == 3;
+    issue(u, 0);
+    if (deep) issue(u + warps, 1);
+    uint32_t slot = 0, fill = deep ? 2 : 1;
 #pragma unroll 1
-    for (; s < a.slices; s += stride, buf ^= 1) {
-        issue(s + stride, buf ^ 1);
-        asm volatile("cp.async.wait_group 1;" ::: "memory");  // this slice's copies have landed
+    for (; u < a.units; u += warps) {
+        __syncwarp();  // every lane has read the slot that is filled next
+        issue(u + (deep ? 2 : 1) * warps, fill);
+        if (++fill == a.depth) fill = 0;
+        if (deep) asm volatile("cp.async.wait_group 2;" ::: "memory");  // this unit's copies
+        else asm volatile("cp.async.wait_group 1;" ::: "memory");
+        __syncwarp();  // ... and the other lanes'
+        const unsigned char *in = ring + slot * kUnit;
+        if (++slot == a.depth) slot = 0;
         float2 v[D], w[D];  // each input and its swapped form (y, x)
+        if (tb == 0) {
 #pragma unroll
-        for (int j = 0; j < D; ++j) {
-            v[j] = stage[(buf * D + j) * 256 + threadIdx.x];
-            w[j] = make_float2(v[j].y, v[j].x);
+            for (int j = 0; j < D; j += 2) {
+                const float4 x = *reinterpret_cast<const float4 *>(
+                    in + (quad ? ((j & 2) ? rd1 : rd0) + uint32_t(j / 4) * 1024u : rd0 + uint32_t(j / 2) * 512u));
+                v[j] = make_float2(x.x, x.y);
+                v[j + 1] = make_float2(x.z, x.w);
+            }
+        } else {
+#pragma unroll
+            for (int j = 0; j < D; ++j)
+                v[j] = *reinterpret_cast<const float2 *>(in + ((j & 1) ? rd1 : rd0) + uint32_t(j / 2) * 512u);
         }
-        float2 *p = psi + base_of(s);
+#pragma unroll
+        for (int j = 0; j < D; ++j) w[j] = make_float2(v[j].y, v[j].x);
+        unsigned char *out = reinterpret_cast<unsigned char *>(psi) + (sbase | unit_base(u));
+        float2 held[4];  // outputs j & ~3 .. j
 #pragma unroll
         for (int j = 0; j < D; ++j) {
             float2 acc = make_float2(0.f, 0.f);
 #pragma unroll
             for (int l = 0; l < D; ++l) {
-                const CEnt &u = a.U[j][l];
-                acc = __ffma2_rn(u.rr, v[l], acc);
-                acc = __ffma2_rn(u.ni, w[l], acc);
+                const CEnt &e = a.U[j][l];
+                acc = __ffma2_rn(e.rr, v[l], acc);
+                acc = __ffma2_rn(e.ni, w[l], acc);
             }
-            p[offs[j]] = acc;
+            held[j & 3] = acc;
+            if (smode == 0) {
+                *reinterpret_cast<float2 *>(out + a.joff[j]) = acc;
+            } else if (j & 1) {
+                const float2 x = held[(j & 3) - 1], y = held[j & 3];
+                if (smode == 1) {
+                    st16(out + a.joff[j - 1], x, y);
+                } else if (smode == 2) {
+                    const float2 send = odd ? x : y;
+                    const float2 recv = make_float2(__shfl_xor_sync(0xffffffffu, send.x, 1),
+                                                    __shfl_xor_sync(0xffffffffu, send.y, 1));
+                    st16(out + a.joff[j - 1], odd ? recv : x, odd ? y : recv);
+                } else if ((j & 3) == 3) {
+                    asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(out + a.joff[j & ~3]),
+                                 "f"(held[0].x), "f"(held[0].y), "f"(held[1].x), "f"(held[1].y), "f"(held[2].x),
+                                 "f"(held[2].y), "f"(held[3].x), "f"(held[3].y)
+                                 : "memory");
+                }
+            }
         }
     }
     asm volatile("cp.async.wait_all;" ::: "memory");
+}
+
+// States of fewer than 32 slices (n < K + 5): one slice per thread, straight from memory.
+template <int K>
+__global__ void k_fused_small(float2 *__restrict__ psi, uint64_t slices, const __grid_constant__ SimtArgs<K> a) {
+    constexpr int D = 1 << K;
+    const uint64_t s = uint64_t(blockIdx.x) * blockDim.x + threadIdx.x;
+    if (s >= slices) return;
+    uint64_t b = s;
+#pragma unroll
+    for (int i = 0; i < K; ++i) b = insert_zero(b, a.t[i]);
+    float2 v[D], w[D];
+#pragma unroll
+    for (int j = 0; j < D; ++j) {
+        v[j] = psi[b + a.joff[j] / 8];
+        w[j] = make_float2(v[j].y, v[j].x);
+    }
+#pragma unroll
+    for (int j = 0; j < D; ++j) {
+        float2 acc = make_float2(0.f, 0.f);
+#pragma unroll
+        for (int l = 0; l < D; ++l) {
+            acc = __ffma2_rn(a.U[j][l].rr, v[l], acc);
+            acc = __ffma2_rn(a.U[j][l].ni, w[l], acc);
+        }
+        psi[b + a.joff[j] / 8] = acc;
+    }
 }
 
 // ---- k_fused_wide<K>: fused 5- to 7-qubit unitaries on FP32 SIMT cores.
@@ -508,8 +627,8 @@ static int simt_attr() {
     int dev = 0;
     cudaGetDevice(&dev);
     if (dev >= 0 && dev < 64 && attr_done[dev]) return RCS_OK;
-    const int smem = 2 * (1 << K) * 256 * int(sizeof(float2));
-    const cudaError_t e = cudaFuncSetAttribute(k_fused_simt<K>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    const cudaError_t e = cudaFuncSetAttribute(k_fused_simt<K>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                               int(8 * kSimtSlots * simt_unit_bytes<K>()));
     if (e != cudaSuccess) return note_launch_error("fused kernel shared-memory attribute", e);
     if (dev >= 0 && dev < 64) attr_done[dev] = true;
     return RCS_OK;
@@ -555,22 +674,41 @@ void simt_build_ops(const Pass &p, uint8_t *out) {
 }
 
 template <int K>
-static int launch_simt_k(float2 *psi, int n, const Pass &p, cudaStream_t st) {
+static int launch_simt_k(float2 *psi, int n, const Pass &p, bool backwards, cudaStream_t st) {
     SimtArgs<K> a;
     const int D = 1 << K;
-    for (int j = 0; j < D; ++j)
+    for (int i = 0; i < K; ++i) a.t[i] = p.t[i];
+    for (int j = 0; j < D; ++j) {
+        a.joff[j] = 0;
+        for (int i = 0; i < K; ++i)
+            if ((j >> i) & 1) a.joff[j] |= 8ull << p.t[i];
         for (int l = 0; l < D; ++l) {
             const cd &u = p.U[size_t(j) * D + l];
             a.U[j][l] = CEnt{make_float2(float(u.real()), float(u.real())), make_float2(-float(u.imag()), float(u.imag()))};
         }
-    for (int i = 0; i < K; ++i) a.t[i] = p.t[i];
-    a.slices = 1ull << (n - K);
-    const int threads = 256;
-    const int smem = 2 * (1 << K) * threads * int(sizeof(float2));
+    }
+    if (n < K + 5) {
+        const uint64_t slices = 1ull << (n - K);
+        k_fused_small<K><<<1, 32, 0, st>>>(psi, slices, a);
+        return check_launch();
+    }
+    std::fill(a.upos, a.upos + 32, int8_t(-1));
+    for (int qb = 0, i = 0; qb < n; ++qb) {
+        if (std::find(p.t, p.t + K, qb) != p.t + K) continue;
+        if (i < 5) a.rpos[i] = int8_t(qb);
+        else a.upos[i - 5] = int8_t(qb);
+        ++i;
+    }
+    const bool quad = K > 1 && p.t[0] == 0 && p.t[1] == 1;
+    for (int c = 0; c < D / 2; ++c)
+        a.coff[c] = quad ? ((c & 1) ? 8ull << a.rpos[4] : 0ull) + a.joff[4 * (c >> 1)] : a.joff[2 * c];
+    a.units = 1ull << (n - K - 5);
+    a.flip = backwards ? uint32_t(a.units - 1) : 0u;
+    a.depth = simt_depth<K>(p.t[0]);
     if (int rc = simt_attr<K>(); rc != RCS_OK) return rc;
-    // persistent: the resident CTAs, never more than the slices need
-    const unsigned grid = grid_for(a.slices, threads, device_sm_count(), simt_blocks_per_sm<K>());
-    k_fused_simt<K><<<grid, threads, smem, st>>>(psi, a);
+    // persistent: the resident CTAs, never more than the units need
+    const unsigned grid = grid_for(a.units, 8, device_sm_count(), simt_blocks_per_sm<K>());
+    k_fused_simt<K><<<grid, 256, 8 * kSimtSlots * simt_unit_bytes<K>(), st>>>(psi, a);
     return check_launch();
 }
 
@@ -589,15 +727,15 @@ static int launch_wide_k(float2 *psi, int n, const Pass &p, const uint8_t *ops, 
     return check_launch();
 }
 
-int launch_pass_simt(void *psi, int n, const Pass &p, const uint8_t *ops, void *stream) {
+int launch_pass_simt(void *psi, int n, const Pass &p, const uint8_t *ops, void *stream, bool backwards) {
     auto st = static_cast<cudaStream_t>(stream);
     auto *s = static_cast<float2 *>(psi);
     if (p.k > n) return RCS_ERR_ARG;
     switch (p.k) {
-        case 1: return launch_simt_k<1>(s, n, p, st);
-        case 2: return launch_simt_k<2>(s, n, p, st);
-        case 3: return launch_simt_k<3>(s, n, p, st);
-        case 4: return launch_simt_k<4>(s, n, p, st);
+        case 1: return launch_simt_k<1>(s, n, p, backwards, st);
+        case 2: return launch_simt_k<2>(s, n, p, backwards, st);
+        case 3: return launch_simt_k<3>(s, n, p, backwards, st);
+        case 4: return launch_simt_k<4>(s, n, p, backwards, st);
         case 5: return launch_wide_k<5>(s, n, p, ops, st);
         case 6: return launch_wide_k<6>(s, n, p, ops, st);
         case 7: return launch_wide_k<7>(s, n, p, ops, st);

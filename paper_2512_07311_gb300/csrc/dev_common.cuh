@@ -3,6 +3,7 @@
 
 #include <cstdint>
 #include <cuda_runtime.h>
+#include <utility>
 
 namespace rcs {
 
@@ -62,6 +63,29 @@ inline unsigned grid_for(uint64_t items, unsigned threads, int sms, int per_sm) 
     uint64_t cap = uint64_t(sms) * uint64_t(per_sm);
     if (need < 1) need = 1;
     return unsigned(need < cap ? need : cap);
+}
+
+// Programmatic dependent launch: a kernel launched with launch_after may start while the
+// kernel before it in the stream still runs (once that one's CTAs have all called
+// grid_trigger or ended), does what needs none of its results, and calls grid_wait before it
+// touches any state: grid_wait returns when that kernel has ended and its stores are visible.
+__device__ __forceinline__ void grid_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+template <class... Params, class... Args>
+inline cudaError_t launch_after(void (*kernel)(Params...), unsigned grid, unsigned block, size_t smem, cudaStream_t st,
+                                Args &&...args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
 }
 
 int device_sm_count();

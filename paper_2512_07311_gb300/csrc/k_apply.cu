@@ -205,6 +205,7 @@ __global__ void __launch_bounds__(256, simt_blocks_per_sm<K>())
     constexpr int D = 1 << K;
     constexpr uint32_t kUnit = simt_unit_bytes<K>();
     extern __shared__ __align__(16) unsigned char simt_smem[];
+    grid_trigger();
     const int lane = threadIdx.x & 31;
     const uint32_t warps = gridDim.x * 8u;
     const int tb = a.t[0] < 5 ? a.t[0] : 5;
@@ -261,6 +262,7 @@ __global__ void __launch_bounds__(256, simt_blocks_per_sm<K>())
     };
     uint32_t u = blockIdx.x * 8u + (threadIdx.x >> 5);
     const bool deep = a.depth == 3;
+    grid_wait();  // the pass before (launch_after)
     issue(u, 0);
     if (deep) issue(u + warps, 1);
     uint32_t slot = 0, fill = deep ? 2 : 1;
@@ -330,6 +332,8 @@ template <int K>
 __global__ void k_fused_small(float2 *__restrict__ psi, uint64_t slices, const __grid_constant__ SimtArgs<K> a) {
     constexpr int D = 1 << K;
     const uint64_t s = uint64_t(blockIdx.x) * blockDim.x + threadIdx.x;
+    grid_trigger();
+    grid_wait();
     if (s >= slices) return;
     uint64_t b = s;
 #pragma unroll
@@ -413,6 +417,7 @@ __global__ void __launch_bounds__(kWideThreads, wide_blocks_per_sm<K>())
     uint64_t *offs = reinterpret_cast<uint64_t *>(buf + (S::Dbl ? 2 : 1) * D * Row);
     const int tid = threadIdx.x;
     const uint64_t slices = a.slices;
+    grid_trigger();
     for (int j = tid; j < D; j += kWideThreads) {
         uint64_t o = 0;
 #pragma unroll
@@ -428,6 +433,7 @@ __global__ void __launch_bounds__(kWideThreads, wide_blocks_per_sm<K>())
         asm volatile("cp.async.commit_group;" ::: "memory");
     }
     __syncthreads();  // offs
+    grid_wait();      // the pass before (launch_after); U came from the host
     const uint64_t ntiles = (slices + T - 1) / T;
     // copy / store walk: slice s = tid % T, rows j = tid / T + (256 / T) i
     const int ws = tid % T, wj = tid / T;
@@ -509,6 +515,8 @@ __global__ void __launch_bounds__(kWideThreads, wide_blocks_per_sm<K>())
 }
 
 __global__ void k_init_zero(float4 *__restrict__ psi4, uint64_t n4) {
+    grid_trigger();
+    grid_wait();
     const uint64_t stride = uint64_t(gridDim.x) * blockDim.x;
     for (uint64_t i = uint64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < n4; i += stride)
         psi4[i] = make_float4(i == 0 ? 1.f : 0.f, 0.f, 0.f, 0.f);
@@ -538,6 +546,8 @@ __global__ void k_expand(float4 *__restrict__ psi4, uint64_t n4, const float2 *_
                          const __grid_constant__ ExpandArgs a) {
     const uint64_t stride = uint64_t(gridDim.x) * blockDim.x;
     const bool pair = a.tmask & 1ull;
+    grid_trigger();
+    grid_wait();
     for (uint64_t f = uint64_t(blockIdx.x) * blockDim.x + threadIdx.x; f < n4; f += stride) {
         const uint64_t i0 = 2 * f;
         float4 out = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -575,17 +585,19 @@ int launch_expand(void *psi, int n, const void *sub, uint64_t tmask, void *strea
         q += len;
     }
     const uint64_t n4 = (1ull << n) / 2;
-    k_expand<<<grid_for(n4, 256, device_sm_count(), 8), 256, 0, static_cast<cudaStream_t>(stream)>>>(
-        static_cast<float4 *>(psi), n4, static_cast<const float2 *>(sub), a);
-    return launch_status("state expansion");
+    const cudaError_t e = launch_after(k_expand, grid_for(n4, 256, device_sm_count(), 8), 256, 0,
+                                       static_cast<cudaStream_t>(stream), static_cast<float4 *>(psi), n4,
+                                       static_cast<const float2 *>(sub), a);
+    return e == cudaSuccess ? RCS_OK : note_launch_error("state expansion", e);
 }
 
 int launch_init_zero(void *psi, int n, void *stream) {
     auto st = static_cast<cudaStream_t>(stream);
     if (n == 0) return RCS_ERR_ARG;
     const uint64_t n4 = (1ull << n) / 2;  // n >= 1: whole float4s
-    k_init_zero<<<grid_for(n4, 256, device_sm_count(), 8), 256, 0, st>>>(static_cast<float4 *>(psi), n4);
-    return check_launch();
+    const cudaError_t e =
+        launch_after(k_init_zero, grid_for(n4, 256, device_sm_count(), 8), 256, 0, st, static_cast<float4 *>(psi), n4);
+    return e == cudaSuccess ? RCS_OK : note_launch_error("zero state", e);
 }
 
 int launch_pass_plain(void *psi, int n, const Pass &p, void *stream) {
@@ -689,8 +701,8 @@ static int launch_simt_k(float2 *psi, int n, const Pass &p, bool backwards, cuda
     }
     if (n < K + 5) {
         const uint64_t slices = 1ull << (n - K);
-        k_fused_small<K><<<1, 32, 0, st>>>(psi, slices, a);
-        return check_launch();
+        const cudaError_t e = launch_after(k_fused_small<K>, 1, 32, 0, st, psi, slices, a);
+        return e == cudaSuccess ? RCS_OK : note_launch_error("fused pass", e);
     }
     std::fill(a.upos, a.upos + 32, int8_t(-1));
     for (int qb = 0, i = 0; qb < n; ++qb) {
@@ -708,8 +720,8 @@ static int launch_simt_k(float2 *psi, int n, const Pass &p, bool backwards, cuda
     if (int rc = simt_attr<K>(); rc != RCS_OK) return rc;
     // persistent: the resident CTAs, never more than the units need
     const unsigned grid = grid_for(a.units, 8, device_sm_count(), simt_blocks_per_sm<K>());
-    k_fused_simt<K><<<grid, 256, 8 * kSimtSlots * simt_unit_bytes<K>(), st>>>(psi, a);
-    return check_launch();
+    const cudaError_t e = launch_after(k_fused_simt<K>, grid, 256, 8 * kSimtSlots * simt_unit_bytes<K>(), st, psi, a);
+    return e == cudaSuccess ? RCS_OK : note_launch_error("fused pass", e);
 }
 
 template <int K>
@@ -723,8 +735,9 @@ static int launch_wide_k(float2 *psi, int n, const Pass &p, const uint8_t *ops, 
     const uint64_t tiles = (a.slices + WideShape<K>::T - 1) / WideShape<K>::T;
     const uint64_t resident = uint64_t(device_sm_count()) * wide_blocks_per_sm<K>();
     const unsigned grid = unsigned(tiles < resident ? tiles : resident);
-    k_fused_wide<K><<<grid, kWideThreads, wide_smem_bytes<K>(), st>>>(psi, reinterpret_cast<const float2 *>(ops), a);
-    return check_launch();
+    const cudaError_t e = launch_after(k_fused_wide<K>, grid, kWideThreads, wide_smem_bytes<K>(), st, psi,
+                                       reinterpret_cast<const float2 *>(ops), a);
+    return e == cudaSuccess ? RCS_OK : note_launch_error("wide fused pass", e);
 }
 
 int launch_pass_simt(void *psi, int n, const Pass &p, const uint8_t *ops, void *stream, bool backwards) {

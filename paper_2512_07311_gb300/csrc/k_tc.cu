@@ -171,7 +171,10 @@ __global__ void __launch_bounds__(kChain ? tc::kChainThreads : tc::kThreads, 1)
 #pragma unroll
     for (int i = 0; i < K; ++i) t[i] = ps.t[i];
 
-    // ---- set-up: operand image, offset table, barriers, tensor memory
+    // ---- set-up: operand image, offset table, barriers, tensor memory. None of it depends on the
+    // pass before, so it overlaps that pass's end (grid_wait): at 19 qubits, where a pass has 64
+    // tiles, most of its 9.6 us were this and the launch itself.
+    if constexpr (!kChain) grid_trigger();
     {
         uint4 *dst = reinterpret_cast<uint4 *>(sm);
         for (int i = threadIdx.x; i < L::kBBytes / 16; i += kThreads) dst[i] = ps.ops[i];
@@ -252,6 +255,7 @@ __global__ void __launch_bounds__(kChain ? tc::kChainThreads : tc::kThreads, 1)
             asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
         }
         tc_fence_before();
+        if constexpr (!kChain) grid_wait();
         __syncthreads();
         tc_fence_after();
     }
@@ -1130,18 +1134,18 @@ static int launch_tc(void *psi, int n, const Pass &p, const void *d_ops, int *d_
     // a short contiguous run and the memory-order variant is faster (158 -> 79 ms for targets 0..5
     // at 34 qubits); for fewer low targets the slice-order variant measured faster.
     cudaStream_t st = static_cast<cudaStream_t>(stream);
+    const size_t smem = tf32 ? Layout<true>::kAlloc : Layout<false>::kAlloc;
+    void (*kernel)(const TcArgs<1>) = nullptr;
     if (sub) {
         if (staged) return RCS_ERR_UNSUPPORTED;  // the sub-state input has a slice-order loader only
-        if (tf32) k_fused_tc<false, true, true, false><<<grid, kThreads, Layout<true>::kAlloc, st>>>(a);
-        else k_fused_tc<false, false, true, false><<<grid, kThreads, Layout<false>::kAlloc, st>>>(a);
+        kernel = tf32 ? k_fused_tc<false, true, true, false> : k_fused_tc<false, false, true, false>;
     } else if (tf32) {
-        if (staged) k_fused_tc<true, true, false, false><<<grid, kThreads, Layout<true>::kAlloc, st>>>(a);
-        else k_fused_tc<false, true, false, false><<<grid, kThreads, Layout<true>::kAlloc, st>>>(a);
+        kernel = staged ? k_fused_tc<true, true, false, false> : k_fused_tc<false, true, false, false>;
     } else {
-        if (staged) k_fused_tc<true, false, false, false><<<grid, kThreads, Layout<false>::kAlloc, st>>>(a);
-        else k_fused_tc<false, false, false, false><<<grid, kThreads, Layout<false>::kAlloc, st>>>(a);
+        kernel = staged ? k_fused_tc<true, false, false, false> : k_fused_tc<false, false, false, false>;
     }
-    return launch_status("tensor-core pass");
+    const cudaError_t e = launch_after(kernel, grid, kThreads, smem, st, a);
+    return e == cudaSuccess ? RCS_OK : note_launch_error("tensor-core pass", e);
 }
 
 int launch_pass_tc(void *psi, int n, const Pass &p, const void *d_ops, int *d_err, void *stream, bool tf32,

@@ -14,8 +14,8 @@
 //    mat-vec reads it as constant operands. 8 * 2^K real flop per amplitude:
 //    HBM-bound up to K = 4 on GB300 (at K = 4 just so: the packed multiply-adds
 //    reach 68 TFLOP/s with nothing else to do, 253 us of a pass of 340).
-//  * k_fused_wide<K>: fused K = 5, 6 or 7 qubit unitaries, a CTA per tile of 128
-//    (K = 5) or 64 slices, U from a device image in shared memory (see below).
+//  * k_fused_wide<K>: fused K = 5, 6 or 7 qubit unitaries, a CTA per tile of 128,
+//    64 or 32 slices, U from a device image in shared memory (see below).
 //    Bound by the FP32 FMA pipe.
 #include <algorithm>
 
@@ -362,33 +362,35 @@ __global__ void k_fused_small(float2 *__restrict__ psi, uint64_t slices, const _
 // operands it is 16 KB at K = 5), and from K = 6 not the parameter space or a thread's
 // registers, so a CTA applies it to a tile of T consecutive slices as a small complex
 // GEMM in shared memory: out[s][j] = sum_l U[j][l] in[s][l], FP32 fused multiply-adds
-// over l in increasing order. U comes from a device image laid out [l][j] (float2 re, im) and is
-// copied into shared memory once per CTA. Each tile is copied in with cp.async into a
-// [j][s] buffer (rows padded by one amplitude), multiplied, written back into the same
-// buffer and stored with the same coalesced [j][s] walk. 8 * 2^K real flop per amplitude
-// (16 to 64 flop/B): past the FP32 ridge, so these passes are bound by the FMA pipe.
+// over l in increasing order. U comes from a device image laid out [l][j] (float2 re, im) and
+// is copied into shared memory once per CTA. 8 * 2^K real flop per amplitude (16 to 64
+// flop/B): past the FP32 ridge, so these passes are bound by the FMA pipe.
+//
+// A warp computes RJ outputs of 32 RS slices, a lane its slices (lane + 32 r): the matrix
+// entries are the same for all lanes, the inputs are neighbouring words, and the outputs go
+// straight to memory in runs of 32 slices. Outputs are packed by twos: the image holds (re_j,
+// re_j+1, im_j, im_j+1), one 16-byte broadcast read, and four packed FP32x2 multiply-adds with
+// (x, x), (-y, -y), (y, y), (x, x) do both outputs' complex multiply-add, per component the same
+// operations in the same order as scalar ones. Two tile buffers let the next tile's copies run
+// under the whole of the current tile's multiply-adds, with one barrier per tile. (Before: 4 x 4
+// and 4 x 8 outputs per thread across lanes, scalar, outputs regrouped through shared memory
+// with three more barriers, and no second buffer at K = 7.) Measured at 27 qubits, before and
+// after, us a pass: K = 5 851-911 and 739-757, K = 6 1371-1419 and 1306-1342, K = 7 2757-2787 and
+// 2450-2484 (46, 53 and 56 TFLOP/s now; packed multiply-adds with nothing else to do reach 68).
 constexpr int kWideThreads = 256;
 
-// Per width: each thread computes RS slices x RJ outputs (slices sg + SG r, outputs
-// jg + JG c; JG x SG = 256 threads), so a tile holds T = SG x RS slices: 4 x 4 on 128
-// slices at K = 5, 4 x 4 and 4 x 8 on 64 slices at K = 6 and 7. Up to K = 6 two tile
-// buffers let the next tile's copies run under the current tile's multiply-adds (the
-// CTAs of an SM otherwise stay in step: all copying, then all multiplying); at K = 7 only
-// one fits beside U. Resident CTAs per SM, by shared memory: three at K = 5 (74 KB), two
-// at K = 6 (99 KB), one at K = 7 (194 KB).
+// Per width: RS slices per lane, RJ outputs per warp; the warps of a group share slices, and
+// the groups of a CTA split a tile's. Resident CTAs per SM, by shared memory: three at K = 5
+// (72 KB), two at K = 6 (96 KB), one at K = 7 (192 KB).
 template <int K>
 struct WideShape {
     static constexpr int D = 1 << K;
-    static constexpr int RS = 4;
-    static constexpr int RJ = K == 7 ? 8 : 4;
-    static constexpr int JG = D / RJ;
-    static constexpr int SG = kWideThreads / JG;
-    static constexpr int T = SG * RS;
-    static constexpr int Row = T + 1;  // buffer row, padded by one amplitude
-    static constexpr bool Dbl = K <= 6;  // two tile buffers: the next tile's copies run under the multiply-adds
+    static constexpr int RS = K == 5 ? 2 : 1;
+    static constexpr int RJ = K == 5 ? 8 : 16;
+    static constexpr int Group = D / RJ;                         // warps of a group
+    static constexpr int T = 32 * RS * (kWideThreads / 32 / Group);  // slices of a tile
     static constexpr int Blocks = K == 5 ? 3 : (K == 6 ? 2 : 1);
-    static constexpr size_t Smem = size_t(D) * D * 8 + (Dbl ? 2 : 1) * size_t(D) * Row * 8 + size_t(D) * 8;
-    static_assert(JG * SG == kWideThreads && T <= kWideThreads && kWideThreads % T == 0, "tile shape");
+    static constexpr size_t Smem = size_t(D) * D * 8 + 2 * size_t(D) * T * 8 + size_t(D) * 8;
 };
 
 template <int K>
@@ -410,11 +412,11 @@ template <int K>
 __global__ void __launch_bounds__(kWideThreads, wide_blocks_per_sm<K>())
     k_fused_wide(float2 *__restrict__ psi, const float2 *__restrict__ ut, const __grid_constant__ WideArgs a) {
     using S = WideShape<K>;
-    constexpr int D = S::D, RS = S::RS, RJ = S::RJ, JG = S::JG, SG = S::SG, T = S::T, Row = S::Row;
+    constexpr int D = S::D, RS = S::RS, RJ = S::RJ, T = S::T;
     extern __shared__ __align__(16) unsigned char wide_smem[];
-    float2 *U = reinterpret_cast<float2 *>(wide_smem);  // [l][j]
-    float2 *buf = U + D * D;                             // [j][Row], twice when double-buffered
-    uint64_t *offs = reinterpret_cast<uint64_t *>(buf + (S::Dbl ? 2 : 1) * D * Row);
+    float2 *U = reinterpret_cast<float2 *>(wide_smem);  // [l][j], packed by two outputs (simt_build_ops)
+    float2 *buf = U + D * D;                             // two of [j][T]
+    uint64_t *offs = reinterpret_cast<uint64_t *>(buf + 2 * D * T);
     const int tid = threadIdx.x;
     const uint64_t slices = a.slices;
     grid_trigger();
@@ -435,10 +437,10 @@ __global__ void __launch_bounds__(kWideThreads, wide_blocks_per_sm<K>())
     __syncthreads();  // offs
     grid_wait();      // the pass before (launch_after); U came from the host
     const uint64_t ntiles = (slices + T - 1) / T;
-    // copy / store walk: slice s = tid % T, rows j = tid / T + (256 / T) i
+    // copy walk: slice s = tid % T, rows j = tid / T + (256 / T) i
     const int ws = tid % T, wj = tid / T;
-    // compute: slices sg + SG r, outputs jg + JG c
-    const int jg = tid % JG, sg = tid / JG;
+    // compute: slices s0 + 32 r, outputs j0 .. j0 + RJ - 1
+    const int s0 = (tid & 31) + (tid >> 5) / S::Group * (32 * RS), j0 = (tid >> 5) % S::Group * RJ;
     const uint32_t buf0 = uint32_t(__cvta_generic_to_shared(buf));
     auto base_of = [&](uint64_t sl) {
         uint64_t b = sl;
@@ -446,70 +448,67 @@ __global__ void __launch_bounds__(kWideThreads, wide_blocks_per_sm<K>())
         for (int i = 0; i < K; ++i) b = insert_zero(b, a.t[i]);
         return b;
     };
-    // copies of tile `tile` into buffer `which` (one commit group per call, possibly empty)
     auto issue = [&](uint64_t tile, int which) {
         const uint64_t sl = tile * T + uint64_t(ws);
         if (tile < ntiles && sl < slices) {
             const uint64_t b = base_of(sl);
-            const uint32_t dst0 = buf0 + uint32_t(which * D * Row) * 8u;
+            const uint32_t dst0 = buf0 + uint32_t(which * D * T) * 8u;
 #pragma unroll 4
             for (int j = wj; j < D; j += kWideThreads / T) {
-                const uint32_t dst = dst0 + uint32_t(j * Row + ws) * 8u;
+                const uint32_t dst = dst0 + uint32_t(j * T + ws) * 8u;
                 asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(dst), "l"(psi + (b | offs[j])) : "memory");
             }
         }
         asm volatile("cp.async.commit_group;" ::: "memory");
     };
     int cur = 0;
-    if (S::Dbl) issue(blockIdx.x, 0);
+    issue(blockIdx.x, 0);
 #pragma unroll 1
-    for (uint64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
-        const uint64_t s = tile * T + uint64_t(ws);
-        const bool live = s < slices;
-        const uint64_t base = base_of(s);
-        if (S::Dbl) {
-            issue(tile + gridDim.x, cur ^ 1);  // that buffer's last stores ended before the last barrier
-            asm volatile("cp.async.wait_group 1;" ::: "memory");
-        } else {
-            issue(tile, 0);
-            asm volatile("cp.async.wait_all;" ::: "memory");
-        }
-        float2 *bt = buf + cur * D * Row;
-        __syncthreads();
-        float2 acc[RS][RJ];
+    for (uint64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x, cur ^= 1) {
+        asm volatile("cp.async.wait_group 0;" ::: "memory");
+        __syncthreads();  // the tile has landed, and every thread is done with the other buffer
+        issue(tile + gridDim.x, cur ^ 1);
+        const float2 *bt = buf + cur * D * T + s0;
+        const float4 *u4 = reinterpret_cast<const float4 *>(U + j0);
+        float2 X[RS][RJ / 2], Y[RS][RJ / 2];  // real and imaginary parts of outputs j, j + 1
 #pragma unroll
         for (int r = 0; r < RS; ++r)
 #pragma unroll
-            for (int c = 0; c < RJ; ++c) acc[r][c] = make_float2(0.f, 0.f);
+            for (int c = 0; c < RJ / 2; ++c) X[r][c] = Y[r][c] = make_float2(0.f, 0.f);
 #pragma unroll 2
         for (int l = 0; l < D; ++l) {
-            float2 x[RS], u[RJ];
+            float2 x[RS];
+            float4 u[RJ / 2];
 #pragma unroll
-            for (int r = 0; r < RS; ++r) x[r] = bt[l * Row + sg + SG * r];
+            for (int r = 0; r < RS; ++r) x[r] = bt[l * T + 32 * r];
 #pragma unroll
-            for (int c = 0; c < RJ; ++c) u[c] = U[l * D + jg + JG * c];
+            for (int c = 0; c < RJ / 2; ++c) u[c] = u4[l * (D / 2) + c];
 #pragma unroll
-            for (int r = 0; r < RS; ++r)
+            for (int r = 0; r < RS; ++r) {
+                const float2 xx = make_float2(x[r].x, x[r].x), yy = make_float2(x[r].y, x[r].y),
+                             ny = make_float2(-x[r].y, -x[r].y);
 #pragma unroll
-                for (int c = 0; c < RJ; ++c) {
-                    acc[r][c].x = fmaf(u[c].x, x[r].x, acc[r][c].x);
-                    acc[r][c].x = fmaf(-u[c].y, x[r].y, acc[r][c].x);
-                    acc[r][c].y = fmaf(u[c].x, x[r].y, acc[r][c].y);
-                    acc[r][c].y = fmaf(u[c].y, x[r].x, acc[r][c].y);
+                for (int c = 0; c < RJ / 2; ++c) {
+                    const float2 re = make_float2(u[c].x, u[c].y), im = make_float2(u[c].z, u[c].w);
+                    X[r][c] = __ffma2_rn(re, xx, X[r][c]);
+                    X[r][c] = __ffma2_rn(im, ny, X[r][c]);
+                    Y[r][c] = __ffma2_rn(re, yy, Y[r][c]);
+                    Y[r][c] = __ffma2_rn(im, xx, Y[r][c]);
                 }
+            }
         }
-        __syncthreads();  // every input read before the buffer takes the outputs
 #pragma unroll
-        for (int r = 0; r < RS; ++r)
+        for (int r = 0; r < RS; ++r) {
+            const uint64_t s = tile * T + uint64_t(s0 + 32 * r);
+            if (s < slices) {
+                float2 *p = psi + base_of(s);
 #pragma unroll
-            for (int c = 0; c < RJ; ++c) bt[(jg + JG * c) * Row + sg + SG * r] = acc[r][c];
-        __syncthreads();
-        if (live) {
-#pragma unroll 4
-            for (int j = wj; j < D; j += kWideThreads / T) psi[base | offs[j]] = bt[j * Row + ws];
+                for (int c = 0; c < RJ / 2; ++c) {
+                    p[offs[j0 + 2 * c]] = make_float2(X[r][c].x, Y[r][c].x);
+                    p[offs[j0 + 2 * c + 1]] = make_float2(X[r][c].y, Y[r][c].y);
+                }
+            }
         }
-        __syncthreads();  // the stores have read the buffer before copies into it are issued
-        if (S::Dbl) cur ^= 1;
     }
     asm volatile("cp.async.wait_all;" ::: "memory");
 }
@@ -673,15 +672,17 @@ int simt_prepare_device() {
 
 size_t simt_ops_bytes(int k) { return k > kSimtParamK ? size_t(8) << (2 * k) : 0; }
 
-// FP32 image of a wide pass: entry (l, j) = U[j][l] as (re, im), l-major.
+// FP32 image of a wide pass, l-major: per l and pair of outputs j, j + 1 (j even) the real
+// parts of U[j][l] and U[j + 1][l], then their imaginary parts.
 void simt_build_ops(const Pass &p, uint8_t *out) {
     const int D = 1 << p.k;
     auto *f = reinterpret_cast<float *>(out);
     for (int l = 0; l < D; ++l)
         for (int j = 0; j < D; ++j) {
             const cd &u = p.U[size_t(j) * D + l];
-            f[2 * (size_t(l) * D + j)] = float(u.real());
-            f[2 * (size_t(l) * D + j) + 1] = float(u.imag());
+            float *at = f + 2 * (size_t(l) * D + (j & ~1)) + (j & 1);
+            at[0] = float(u.real());
+            at[2] = float(u.imag());
         }
 }
 

@@ -89,32 +89,53 @@ struct BArgs {
     long long skip_item;  // an item whose completion is never published (fault test), or -1
 };
 
-// offs: the 2^K target offsets in shared memory, read back through a volatile
-// pointer at each use so they are not held in registers across the mat-vec.
+// Slices [s_begin, s_end) of one pass. A thread takes kPer slices at once, kThreads apart, so
+// that one read of a matrix entry from shared memory serves kPer * 4 multiply-adds: with one
+// slice these reads (one per 4) bound the kernel at width 4, 28 TFLOP/s; two slices' inputs
+// fit the registers up to width 4. offs: the 2^K target offsets in shared memory, read back
+// through a volatile pointer at each use so they are not held in registers across the mat-vec.
 template <int K>
 __device__ __forceinline__ void apply_items(float2 *__restrict__ psi, const int *t, const float4 *sU,
                                             const volatile uint64_t *offs, uint64_t s_begin, uint64_t s_end) {
     constexpr int D = 1 << K;
+    constexpr int kPer = K <= 4 ? 2 : 1;
 #pragma unroll 1
-    for (uint64_t s = s_begin + threadIdx.x; s < s_end; s += kThreads) {
-        uint64_t base = s;
+    for (uint64_t s = s_begin + threadIdx.x; s < s_end; s += uint64_t(kPer) * kThreads) {
+        float2 *p[kPer];
+        float2 v[kPer][D];
 #pragma unroll
-        for (int i = 0; i < K; ++i) base = insert_zero(base, t[i]);
-        float2 v[D];
+        for (int k = 0; k < kPer; ++k) {  // past the end: the first slice again, not stored
+            uint64_t base = s + uint64_t(k) * kThreads < s_end ? s + uint64_t(k) * kThreads : s;
 #pragma unroll
-        for (int j = 0; j < D; ++j) v[j] = __ldcg(psi + base + offs[j]);
+            for (int i = 0; i < K; ++i) base = insert_zero(base, t[i]);
+            p[k] = psi + base;
+        }
 #pragma unroll
         for (int j = 0; j < D; ++j) {
-            float2 acc = make_float2(0.f, 0.f);
+            const uint64_t o = offs[j];
+#pragma unroll
+            for (int k = 0; k < kPer; ++k) v[k][j] = __ldcg(p[k] + o);
+        }
+        const bool both = kPer > 1 && s + kThreads < s_end;
+#pragma unroll
+        for (int j = 0; j < D; ++j) {
+            float2 acc[kPer];
+#pragma unroll
+            for (int k = 0; k < kPer; ++k) acc[k] = make_float2(0.f, 0.f);
 #pragma unroll
             for (int l = 0; l < D; ++l) {
                 const float4 u = sU[j * D + l];
-                acc.x = fmaf(u.x, v[l].x, acc.x);
-                acc.x = fmaf(u.z, v[l].y, acc.x);
-                acc.y = fmaf(u.x, v[l].y, acc.y);
-                acc.y = fmaf(u.y, v[l].x, acc.y);
+#pragma unroll
+                for (int k = 0; k < kPer; ++k) {
+                    acc[k].x = fmaf(u.x, v[k][l].x, acc[k].x);
+                    acc[k].x = fmaf(u.z, v[k][l].y, acc[k].x);
+                    acc[k].y = fmaf(u.x, v[k][l].y, acc[k].y);
+                    acc[k].y = fmaf(u.y, v[k][l].x, acc[k].y);
+                }
             }
-            __stcg(psi + base + offs[j], acc);
+            const uint64_t o = offs[j];
+            __stcg(p[0] + o, acc[0]);
+            if (both) __stcg(p[kPer - 1] + o, acc[kPer - 1]);
         }
     }
 }

@@ -619,8 +619,10 @@ def main():
     stages = int(info["prefix_stages"])
     fused = prefix > 0 and full_passes == passes - prefix - 1
     setup = 1 + max(stages - 1, 0) + (0 if (prefix == 0 or fused) else 1)
-    gpu_launches = (passes - pairs) + setup + 1 + 3 + 6 + 2
-    bytes_per_launch = 16.0 * 2.0**n
+    # BF16x3 passes on 24 or more qubits run chained, two or three in one launch: count three
+    chained = args.precision == "bf16x3" and not pairs and n >= 24
+    gpu_launches = (-(-(passes - pairs) // 3) if chained else passes - pairs) + setup + 1 + 3 + 6 + 2
+    bytes_per_launch = 16.0 * 2.0**n  # of one pass; chained passes share one trip through HBM
     achieved = bytes_per_launch / t_pass_s / 1e9
     # traffic: DRAM bytes per launch from an ncu capture of the same kernel (None for a kernel
     # not captured since it last changed)
@@ -631,6 +633,13 @@ def main():
                 "kernel": "k_pair_tc (two unitaries per launch)" if pairs else "k_fused_tc", "peak_src": peaks["src"],
                 "algorithmic_bytes_per_launch": bytes_per_launch, "launches_per_step": full_passes,
                 "mean_launch_ms": t_pass_s * 1e3}
+    if chained:
+        # per pass, as if each made its own trip: above 1 because two or three share one through L2
+        # (HBM itself moves 1/2 to 1/3 of these bytes; the SM's tile pipeline is the bound)
+        roofline.update({"bound": "sm pipeline", "kernel": "k_fused_tc (chained passes)", "traffic": None,
+                         "traffic_src": None,
+                         "note": "bytes and time are per pass; 2 or 3 passes share one trip through HBM, so "
+                                 "frac compares with passes that stream from HBM and may exceed 1"})
 
     # end to end through the host-buffer API: gate list in, samples out, samples in, XEB out
     e2e_ms = []

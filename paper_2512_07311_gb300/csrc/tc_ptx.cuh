@@ -76,12 +76,14 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
     return true;
 }
 
-// Warp-uniform bounded wait: lane 0 polls (with the time limit), the outcome is
-// broadcast, then every lane performs its own (now immediately successful)
-// acquiring test so the whole warp is ordered after the phase. The phase cannot
+// Warp-uniform bounded wait. Every lane tests the phase first, which mostly is complete
+// (going straight to lane 0's loop cost TF32x3 passes 4 to 14% of their time in L2). Else
+// lane 0 polls (with the time limit), the outcome is broadcast, then every lane performs its
+// own (now immediately successful) acquiring test so the whole warp is ordered after the phase. The phase cannot
 // move on before this warp arrives on its own barrier, so the test cannot miss it.
 template <bool kSuspend>
 __device__ __forceinline__ bool warp_wait(uint32_t bar, uint32_t parity, volatile int *abort_flag, long long limit) {
+    if (__all_sync(0xffffffffu, kSuspend ? mbar_try_wait_suspend(bar, parity) : mbar_try_wait(bar, parity))) return true;
     int ok = 1;
     if ((threadIdx.x & 31) == 0) ok = mbar_wait<kSuspend>(bar, parity, abort_flag, limit) ? 1 : 0;
     ok = __shfl_sync(0xffffffffu, ok, 0);

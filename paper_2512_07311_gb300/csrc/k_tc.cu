@@ -112,7 +112,7 @@ __device__ __forceinline__ uint32_t swz(uint32_t c) { return c ^ ((c >> 6) & 15u
 // targets and the lowest qubits, so every pass maps a chunk to itself. CTA b works on pass
 // b mod npass; the CTAs of a pass take its tiles in chunk order, and a pass starts a chunk
 // once the pass before it has stored all of it. A chunk then still sits in L2: with chunks
-// of 4 to 16 MB and a window of 64 to 80 MB between passes, the first pass reads HBM, the
+// of 8 or 16 MB and a window of 64 to 80 MB between passes, the first pass reads HBM, the
 // last one's stores go back to it, and all else runs at L2's rate: at 27 qubits a pair of
 // passes takes 458 us against 2 x 323 one after the other (where HBM runs at its peak), and
 // the SM's own pipeline (2.1 us per tile: 1.5 without any copies and stores) is the bound.

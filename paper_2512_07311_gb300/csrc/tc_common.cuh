@@ -27,10 +27,11 @@ constexpr int kChainThreads = kThreads + 64;    // two more warps order the chun
 // From 128 MB a state no longer stays in L2 from one pass to the next (two passes at 24 qubits:
 // 87 us as a chain, 95 one after the other; at 23 qubits 57 against 47).
 constexpr int kChainMinQubits = 24;
-// A chunk of 4 MB keeps the CTAs of a pass busy for about one tile each. The larger it is, the
-// fewer of them fit the window below; two passes need chunks of up to 2^19 amplitudes, three
-// mostly 2^19 to 2^21.
-constexpr int kChunkMinLog2 = 19;
+// A chunk of 8 MB gives the CTAs of a pass one or two tiles each. The larger it is, the fewer of
+// them fit the window below; two passes need chunks of up to 2^19 amplitudes, three mostly 2^19
+// to 2^21. Measured with chunks of at least 2^18 / 2^19 / 2^20 / 2^21: the 30-qubit, 14-cycle
+// circuit 35.6 / 32.9 / 32.1 / 32.9 ms, the 27-qubit, 20-cycle one 5.72 / 5.23 / 5.19 / 5.31.
+constexpr int kChunkMinLog2 = 20;
 constexpr int kChunkMaxLog2[kChainMax + 1] = {0, 0, 21, 20};
 // Distance between two passes of a chain. The tiles in flight in both (about 4 per SM each) and
 // the counters' round trip take some 70 MB; beyond about 80 MB for a pair and 64 MB a step for

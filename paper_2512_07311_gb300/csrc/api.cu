@@ -478,7 +478,7 @@ int run_substages(const Plan &plan, const std::vector<SubStage> &stages, void *p
         const SubStage &st = stages[si];
         const int m = std::popcount(st.tmask);
         uint8_t *next = buf;
-        buf += size_t(8) << m;
+        buf += substate_stride(m);
         if (cur == nullptr) {
             if (launch_init_zero(next, m, stream) != RCS_OK) return RCS_ERR_CUDA;
         } else {  // the previous sub-state's qubits, numbered inside this one

@@ -618,7 +618,7 @@ bool persistent_steps(const InstHost &h, std::vector<BtcStep> *out) {
         for (const SubStage &st : h.stages) {
             const int m = std::popcount(st.tmask);
             void *next = buf;
-            buf += size_t(8) << m;
+            buf += substate_stride(m);
             if (st.count == 0) continue;
             if (m < kTcK + 7) return false;
             uint64_t inner = 0;  // the previous sub-state's qubits, numbered inside this one

@@ -136,7 +136,9 @@ struct SubStage {
     uint64_t tmask = 0;        // qubits of the sub-state (cumulative over the stages)
 };
 int plan_stages(const Plan &plan, std::vector<SubStage> *stages);
-// Device bytes of the sub-state buffers of the stages (one after another).
+// Device bytes of a stage's sub-state of m qubits (whole 256-byte lines: the passes move up to
+// 32 aligned bytes at a time), and of the buffers of the stages (one after another).
+inline size_t substate_stride(int m) { return m < 5 ? size_t(256) : size_t(8) << m; }
 size_t substage_bytes(const std::vector<SubStage> &stages);
 // Runs the stages of a plan from |0...0> into psi (2^n amplitudes): reset of the first
 // sub-state, its passes, an expansion into the next sub-state, ..., and either an

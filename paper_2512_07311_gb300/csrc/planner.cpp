@@ -1062,7 +1062,7 @@ int plan_stages(const Plan &plan, std::vector<SubStage> *stages) {
 
 size_t substage_bytes(const std::vector<SubStage> &stages) {
     size_t b = 0;
-    for (const SubStage &s : stages) b += size_t(8) << std::popcount(s.tmask);
+    for (const SubStage &s : stages) b += substate_stride(std::popcount(s.tmask));
     return b;
 }
 

@@ -13,20 +13,20 @@
 // 2^-17 relative, is dropped), accumulated in FP32 in tensor memory.
 //
 // Data flow per CTA (persistent, one CTA per SM, 17 warps):
-//   warps 0-7  (loaders):  cp.async 8-byte copies of a tile's amplitudes into a
-//              shared-memory stage (two tiles in flight), then split each amplitude
-//              into bf16x2 hi and lo words and write them to tensor memory with
-//              tcgen05.st: the slice's 64 amplitudes become row s of the A operand
-//              (A is read by the MMA straight from TMEM, lane = slice).
+//   warps 0-7  (loaders):  16-byte cp.async copies of a tile's amplitudes into the
+//              warp's own ring of units in shared memory (up to 2.5 tiles in flight),
+//              then split each amplitude into bf16x2 hi and lo words and write them to
+//              tensor memory with tcgen05.st: the slice's 64 amplitudes become row s of
+//              the A operand (A is read by the MMA straight from TMEM, lane = slice).
 //   warp 16    (MMA):      one thread issues the 24 MMAs of a tile (B = R^T from
 //              shared memory, 128-byte swizzled, K-major) and commits to an mbarrier.
 //   warps 8-15 (epilogue): tcgen05.ld of the FP32 accumulator rows (lane = slice)
-//              and coalesced 8-byte stores of the new amplitudes, in place.
+//              and coalesced 8- to 32-byte stores of the new amplitudes, in place.
 // Tensor memory holds two buffers of {D: 128 cols, A_hi: 64 cols, A_lo: 64 cols},
 // so loading tile i+1, the MMAs of tile i and the stores of tile i-1 overlap.
-// Lanes of a warp always take 32 consecutive slices, so every global load and store
-// instruction walks consecutive addresses along the lowest non-target qubits; with
-// the lowest target on bit 0 or 1 the stores are 16 bytes wide (see the epilogue).
+// A warp always takes 32 consecutive slices, so every global load and store instruction
+// walks consecutive addresses along the lowest qubits, those of low targets included
+// (see the slice-order loader and epilogue).
 //
 // Variants (template parameters):
 //   kStaged: loads and stores walk the tile in memory order through a swizzled stage
@@ -35,7 +35,8 @@
 //            Im y = Xr Ui^T + Xi Ur^T: 48 MMAs of M = N = 128, K = 8 per tile, B images
 //            [Ur; Ui] and [-Ui; Ur] as windows of one [-Ui; Ur; Ui] image per split;
 //   kSub:    the input comes from a compact sub-state (the state is |0> on the qubits
-//            outside it), so the pass also expands that sub-state into the full state.
+//            outside it), so the pass also expands that sub-state into the full state;
+//   kChain:  two or three consecutive BF16 passes in one launch, through L2.
 //
 // Every wait is bounded (about one second of SM clock); on expiry the kernel raises
 // an error bit, drains its own MMAs and copies, frees its tensor memory and returns.
@@ -97,9 +98,9 @@ struct TcArgs {
 // differ only in slice bits (TMEM-side rows) spread over the shared-memory banks.
 __device__ __forceinline__ uint32_t swz(uint32_t c) { return c ^ ((c >> 6) & 15u); }
 
-// kStaged = false: lanes of a loader or epilogue warp take 32 consecutive slices
-// and move 8 bytes each straight between global memory and the stage / registers;
-// coalesced when no target is below qubit 5 (the slices then sit side by side).
+// kStaged = false: a loader or epilogue warp takes 32 consecutive slices and moves them
+// straight between global memory and its ring / registers (the sub-state input 8 bytes
+// per lane, all else 16 to 32 bytes in the order of the index bits).
 // kStaged = true: for passes with low targets, loads and stores walk the tile in
 // memory order (32 consecutive amplitudes per warp instruction) through the
 // swizzled shared-memory stage, which also carries the outputs back out.
@@ -116,8 +117,9 @@ __device__ __forceinline__ uint32_t swz(uint32_t c) { return c ^ ((c >> 6) & 15u
 // last one's stores go back to it, and all else runs at L2's rate: at 27 qubits a pair of
 // passes takes 458 us against 2 x 323 one after the other (where HBM runs at its peak), and
 // the SM's own pipeline (2.1 us per tile: 1.5 without any copies and stores) is the bound.
-// TF32x3 tiles take the SM longer than HBM needs for them, and chains of them measured slower. Two more warps keep the
-// order, so that the loaders and the epilogue never wait for L2:
+// TF32x3 tiles take the SM as long as HBM does, and chains of them measured slower (375
+// against 350 us a pass). Two more warps keep the order, so that the loaders and the
+// epilogue never wait for L2:
 //   warp 17 polls the chunk counters of the passes before and after this CTA's, and tells
 //           the loaders in shared memory how many chunks they may start (the next pass holds
 //           this one back to `window` chunks ahead of it, so a chunk is read while in L2);

@@ -39,7 +39,8 @@ constexpr int kChunkMaxLog2[kChainMax + 1] = {0, 0, 21, 20};
 // 56 / 72 / 80 / 96 / 128 MB 301 / 259 / 233 / 229 / 248 / 288; threes with 20 / 32 / 48 / 64 MB
 // 416 / 289 / 243 / 230.
 constexpr uint64_t kChainWindowBytes[kChainMax + 1] = {0, 0, uint64_t(80) << 20, uint64_t(64) << 20};
-// Time of a chain in passes of one launch each (350 us before, 229 a pass in pairs and threes).
+// Time of a chain in passes of one launch each, for splitting a sequence: pairs and threes take
+// about 0.7 a pass (229 against 328 us at 27 qubits), a pass left over a whole one.
 constexpr double kChainCost[kChainMax + 1] = {0, 1.0, 1.36, 2.06};
 constexpr int kOpBytes = NR * KR * 2;                          // one bf16 operand image: 32 KB
 constexpr int kStageBytes = D * M * 8;                         // one tile of complex64: 64 KB

@@ -40,7 +40,7 @@ constexpr int kChunkMaxLog2[kChainMax + 1] = {0, 0, 21, 20};
 // 416 / 289 / 243 / 230.
 constexpr uint64_t kChainWindowBytes[kChainMax + 1] = {0, 0, uint64_t(80) << 20, uint64_t(64) << 20};
 // Time of a chain in passes of one launch each, for splitting a sequence: pairs and threes take
-// about 0.7 a pass (229 against 328 us at 27 qubits), a pass left over a whole one.
+// about 0.7 a pass (229 to 238 against 323 us at 27 qubits), a pass left over a whole one.
 constexpr double kChainCost[kChainMax + 1] = {0, 1.0, 1.36, 2.06};
 constexpr int kOpBytes = NR * KR * 2;                          // one bf16 operand image: 32 KB
 constexpr int kStageBytes = D * M * 8;                         // one tile of complex64: 64 KB

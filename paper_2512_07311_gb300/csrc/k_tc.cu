@@ -505,7 +505,11 @@ __global__ void __launch_bounds__(kChain ? tc::kChainThreads : tc::kThreads, 1)
                     v = __shfl_sync(0xffffffffu, v, 0);
                     if (c < v) {
                         chunks_open = v;
-                        __threadfence_block();  // the copies below come after the counters that warp 17 saw
+                        // the copies below come after the counters that warp 17 saw: the fence orders
+                        // lane 0's read of the limit, the barrier the other lanes' copies behind that
+                        // (the shuffle hands the value on, but orders no memory)
+                        __threadfence_block();
+                        __syncwarp();
                         return true;
                     }
                     if (!block) return false;

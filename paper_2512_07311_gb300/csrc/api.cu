@@ -771,7 +771,8 @@ int rcs_apply_circuit(rcs_ctx *c, const rcs_gate *gates, size_t n_gates) {
 }
 
 namespace {
-// Largest |(U U^H - 1)[r][c]| of a d x d matrix (row-major, interleaved). U U^H is Hermitian, so
+// Largest |(U U^H - 1)[r][c]| of a d x d matrix (row-major, interleaved); infinite if an entry of
+// U is a NaN or an infinity (row r of U U^H then has one on the diagonal). U U^H is Hermitian, so
 // only c >= r is formed, a row of it at a time from the transposed real and imaginary parts:
 // the inner loop runs over neighbouring columns (vector instructions). The complex triple loop
 // that came before took 2 ms at d = 128, more than a pass of a 26-qubit state.
@@ -796,8 +797,11 @@ double unitarity_error(int d, const double *u) {
                 pi[c] += ai * br[c] - ar * bi[c];
             }
         }
-        for (size_t c = r; c < D; ++c)
-            worst = std::max(worst, std::hypot(sr[c] - (r == c ? 1.0 : 0.0), si[c]));
+        for (size_t c = r; c < D; ++c) {
+            const double e = std::hypot(sr[c] - (r == c ? 1.0 : 0.0), si[c]);
+            if (!std::isfinite(e)) return INFINITY;  // a NaN would pass every comparison with `worst`
+            worst = std::max(worst, e);
+        }
     }
     return worst;
 }

@@ -27,7 +27,9 @@ static double unitarity_defect(const cd *m, int d) {
         for (int c = 0; c < d; ++c) {
             cd s = 0.0;
             for (int l = 0; l < d; ++l) s += m[r * d + l] * std::conj(m[c * d + l]);
-            worst = std::fmax(worst, std::abs(s - (r == c ? 1.0 : 0.0)));
+            const double e = std::abs(s - (r == c ? 1.0 : 0.0));
+            if (!std::isfinite(e)) return INFINITY;  // fmax would drop a NaN
+            worst = std::fmax(worst, e);
         }
     return worst;
 }

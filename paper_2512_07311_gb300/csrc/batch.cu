@@ -766,6 +766,18 @@ int capture(rcs_batch *b) {
     return RCS_OK;
 }
 
+// Makes `dev` the current device for as long as it lives.
+struct OnDevice {
+    int prev = 0;
+    explicit OnDevice(int dev) {
+        cudaGetDevice(&prev);
+        cudaSetDevice(dev);
+    }
+    ~OnDevice() { cudaSetDevice(prev); }
+    OnDevice(const OnDevice &) = delete;
+    OnDevice &operator=(const OnDevice &) = delete;
+};
+
 }  // namespace
 
 extern "C" {
@@ -1030,6 +1042,8 @@ int rcs_batch_state_read(rcs_batch *b, size_t i, uint64_t first, uint64_t count,
     // order (2^16 amplitudes rearranged on the host took 1 ms; the copy takes 0.05)
     const BitMap m = plan_to_stored(h.plan);
     const uint64_t piece = std::min<uint64_t>(count, uint64_t(1) << 23);
+    // the scratch and the kernel belong on the batch's device (the copies find it by themselves)
+    const OnDevice here(b->dev);
     void *scratch = nullptr;
     if (cudaMalloc(&scratch, piece * 8) == cudaSuccess) {
         int rc = RCS_OK;

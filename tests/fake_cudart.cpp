@@ -33,6 +33,11 @@ std::map<const void *, std::string> &kernels() {
     return m;
 }
 
+std::map<const void *, void *> &variables() {
+    static std::map<const void *, void *> m;
+    return m;
+}
+
 struct Config {
     dim3 grid, block;
     size_t smem;
@@ -103,7 +108,9 @@ void __cudaRegisterFunction(void **, const char *fun, char *, const char *name, 
                             int *) {
     kernels()[fun] = name;
 }
-void __cudaRegisterVar(void **, char *, char *, const char *, int, size_t, int, int) {}
+void __cudaRegisterVar(void **, char *var, char *, const char *, int, size_t size, int, int) {
+    variables()[var] = std::calloc(1, size);
+}
 unsigned __cudaPushCallConfiguration(dim3 grid, dim3 block, size_t smem, struct CUstream_st *stream) {
     g_config.push_back({grid, block, smem, stream});
     return 0;
@@ -161,9 +168,9 @@ cudaError_t cudaOccupancyMaxActiveBlocksPerMultiprocessorWithFlags(int *n, const
     return cudaSuccess;
 }
 cudaError_t cudaDeviceSynchronize() { return cudaSuccess; }
-cudaError_t cudaGetSymbolAddress(void **p, const void *) {
-    *p = nullptr;
-    return note(cudaErrorInvalidSymbol);
+cudaError_t cudaGetSymbolAddress(void **p, const void *var) {
+    *p = variables().count(var) ? variables()[var] : nullptr;
+    return note(*p ? cudaSuccess : cudaErrorInvalidSymbol);
 }
 
 // ---- memory

@@ -545,11 +545,14 @@ int launch_pass_range(const Plan &plan, void *psi, int n, size_t first, size_t e
                 ps[j] = &shape[i - first + size_t(j)];
                 ops[j] = d_ops + plan.tc_offset[i + size_t(j)];
             }
-            if (launch_chain_tc(psi, n, ps, ops, count, chain_sync, d_err, stream, backwards) != RCS_OK)
-                return RCS_ERR_CUDA;
-            *launches += count;
-            i += size_t(count);
-            continue;
+            const int rc = launch_chain_tc(psi, n, ps, ops, count, chain_sync, d_err, stream, backwards);
+            if (rc == RCS_OK) {
+                *launches += count;
+                i += size_t(count);
+                continue;
+            }
+            if (rc != RCS_ERR_UNSUPPORTED) return RCS_ERR_CUDA;
+            chain.clear();  // its CTAs cannot be resident together here: single passes from now on
         }
         const Pass &p = at(i, c0);
         if (plan_pairs_at(plan, i, end, n) && plan.pair_offset.size() == plan.passes.size() &&

@@ -182,7 +182,10 @@ int launch_pass_tc_from_sub(void *psi, int n, const Pass &p, const void *d_ops, 
 // Chains: 2 or 3 consecutive BF16x3 tensor-core passes in one launch, the state making one trip
 // through HBM (k_tc.cu). tc_chain_lengths splits a sequence of passes on n qubits: entry i
 // is the number of passes of the group that starts at i. `sync` is scratch of
-// tc_chain_sync_bytes(n) device bytes (0: no chains at that size), cleared by each launch.
+// tc_chain_sync_bytes(n) device bytes (0: no chains at that size), cleared by each launch. A
+// chain needs its CTAs resident together: launch_chain_tc gives RCS_ERR_UNSUPPORTED, with nothing
+// run, where the process has fewer SMs than the device reports (an MPS share, a green context);
+// the passes then run one launch each.
 size_t tc_chain_sync_bytes(int n);
 std::vector<int> tc_chain_lengths(const std::vector<Pass> &passes, int n, bool tf32);
 int launch_chain_tc(void *psi, int n, const Pass *const *p, const void *const *d_ops, int count, uint32_t *sync,

@@ -1216,6 +1216,7 @@ int launch_chain_tc(void *psi, int n, const Pass *const *p, const void *const *d
     if (count < 2 || count > kChainMax || n < kChainMinQubits || !sync) return RCS_ERR_ARG;
     const uint64_t C = chain_chunk(p, count, n);
     if (C == 0) return RCS_ERR_ARG;
+    if (device_sm_count() < count) return RCS_ERR_UNSUPPORTED;  // each pass needs a CTA of its own
     if (int rc = tc_prepare_device(); rc != RCS_OK) return rc;
     TcArgs<kChainMax> a;
     std::memset(&a, 0, sizeof(a));
@@ -1245,6 +1246,10 @@ int launch_chain_tc(void *psi, int n, const Pass *const *p, const void *const *d
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     const cudaError_t e = cudaLaunchKernelEx(&cfg, k_fused_tc<false, false, false, true>, a);
+    if (e == cudaErrorCooperativeLaunchTooLarge || e == cudaErrorNotSupported) {
+        cudaGetLastError();
+        return RCS_ERR_UNSUPPORTED;
+    }
     return e == cudaSuccess ? RCS_OK : note_launch_error("chained tensor-core passes", e);
 }
 

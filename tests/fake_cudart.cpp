@@ -139,7 +139,7 @@ cudaError_t cudaGetLastError() {
 }
 const char *cudaGetErrorString(cudaError_t e) { return e == cudaSuccess ? "no error" : "stand-in error"; }
 cudaError_t cudaGetDeviceCount(int *n) {
-    *n = 2;
+    *n = 3;
     return cudaSuccess;
 }
 cudaError_t cudaGetDevice(int *d) {
@@ -147,7 +147,7 @@ cudaError_t cudaGetDevice(int *d) {
     return cudaSuccess;
 }
 cudaError_t cudaSetDevice(int d) {
-    if (d < 0 || d > 1) return note(cudaErrorInvalidDevice);
+    if (d < 0 || d > 2) return note(cudaErrorInvalidDevice);
     g_device = d;
     return cudaSuccess;
 }

@@ -422,6 +422,7 @@ namespace rcs {
 thread_local std::string g_launch_err;
 
 int note_launch_error(const char *what, cudaError_t e) {
+    cudaGetLastError();  // the runtime keeps e too: the next call's check would find it again
     g_launch_err = std::string(what) + ": " + cudaGetErrorString(e);
     return RCS_ERR_CUDA;
 }

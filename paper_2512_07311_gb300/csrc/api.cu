@@ -311,9 +311,9 @@ BitMap to_stored(const rcs_ctx *c) {
 // Brings the stored state back to the identity layout (the amplitudes move unchanged).
 int restore_layout(rcs_ctx *c) {
     if (!c->zero_pending) {  // |0...0> is the same in any layout
+        c->sums_valid = false;
         if (launch_restore_layout(c->psi, c->n, c->phys_of, c->stream) != RCS_OK)
             return fail(c, RCS_ERR_CUDA, "layout change: " + take_launch_error());
-        c->sums_valid = false;
     }
     set_identity_layout(c);
     return RCS_OK;

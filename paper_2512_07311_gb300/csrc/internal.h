@@ -121,9 +121,9 @@ int launch_init_zero(void *psi, int n, void *stream);
 int launch_expand(void *psi, int n, const void *sub, uint64_t tmask, void *stream);
 // Layout changes (k_layout.cu). launch_restore_layout: psi, whose circuit qubit q is stored
 // at index bit phys_of[q], is put into the identity layout in place (amplitudes move
-// unchanged). launch_read_mapped: out[i] = psi[map(first + i)] for count amplitudes (out on
-// the device).
-int launch_restore_layout(void *psi, int n, const int *phys_of, void *stream);
+// unchanged); phys_of follows the passes launched, so a failure leaves what psi will hold.
+// launch_read_mapped: out[i] = psi[map(first + i)] for count amplitudes (out on the device).
+int launch_restore_layout(void *psi, int n, int *phys_of, void *stream);
 int launch_read_mapped(const void *psi, uint64_t first, uint64_t count, const BitMap &map, void *out, void *stream);
 
 // Leading passes of a fused plan that a run from |0...0> can do on compact

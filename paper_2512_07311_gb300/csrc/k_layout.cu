@@ -115,7 +115,7 @@ static int launch_permute(void *psi, int n, const int *m, cudaStream_t st) {
     return launch_status("layout permutation");
 }
 
-int launch_restore_layout(void *psi, int n, const int *phys_of, void *stream) {
+int launch_restore_layout(void *psi, int n, int *phys_of, void *stream) {
     int phys[64], log_of[64], m[64];
     for (int q = 0; q < n; ++q) {
         phys[q] = phys_of[q];
@@ -128,6 +128,7 @@ int launch_restore_layout(void *psi, int n, const int *phys_of, void *stream) {
     auto flush = [&]() {
         int rc = RCS_OK;
         if (moved != 1) rc = launch_permute(psi, n, m, static_cast<cudaStream_t>(stream));
+        if (rc == RCS_OK) std::copy(phys, phys + n, phys_of);
         for (int q = 0; q < n; ++q) m[q] = q;
         moved = 1;
         return rc;

@@ -225,6 +225,11 @@ int rcs_plan_pass(const rcs_plan *plan, size_t i, int32_t *k, int32_t *targets, 
  * those passes to finish. */
 int rcs_last_pass_timing(rcs_ctx *ctx, float *ms, int64_t *full_passes);
 
+/* Kernel launches of the last rcs_apply_circuit, rcs_apply_unitaries or rcs_plan_run on this
+ * context (the zero fill, sub-state passes and expansions included), and how many of
+ * them ran a chain of two or three passes. */
+int rcs_last_run_launches(rcs_ctx *ctx, int64_t *kernels, int64_t *chains);
+
 /* Uploads the plan's pass table and matrices to the device of ctx (once per plan
  * and context; later calls are no-ops). */
 int rcs_plan_upload(rcs_ctx *ctx, rcs_plan *plan);

@@ -79,6 +79,7 @@ SIGNATURES = [
     ("rcs_plan_pass", ctypes.c_int, [_P, ctypes.c_size_t, _i32p, _i32p, _f64p]),
     ("rcs_plan_upload", ctypes.c_int, [_P, _P]),
     ("rcs_last_pass_timing", ctypes.c_int, [_P, ctypes.POINTER(ctypes.c_float), ctypes.POINTER(ctypes.c_int64)]),
+    ("rcs_last_run_launches", ctypes.c_int, [_P, ctypes.POINTER(ctypes.c_int64), ctypes.POINTER(ctypes.c_int64)]),
     ("rcs_plan_run", ctypes.c_int, [_P, _P]),
     ("rcs_plan_destroy", None, [_P]),
     ("rcs_amplitudes", ctypes.c_int, [_P, _u64p, ctypes.c_size_t, _f64p]),
@@ -272,6 +273,13 @@ def rcs_last_pass_timing(ctx):
     ms, n = ctypes.c_float(), ctypes.c_int64()
     _check(load().rcs_last_pass_timing(ctx, ctypes.byref(ms), ctypes.byref(n)), ctx)
     return ms.value, n.value
+
+
+def rcs_last_run_launches(ctx):
+    """(kernel launches, chains of passes among them) of the last run on ctx."""
+    k, c = ctypes.c_int64(), ctypes.c_int64()
+    _check(load().rcs_last_run_launches(ctx, ctypes.byref(k), ctypes.byref(c)), ctx)
+    return k.value, c.value
 
 
 def rcs_plan_upload(ctx, plan):

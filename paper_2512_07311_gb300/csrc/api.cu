@@ -48,6 +48,7 @@ struct rcs_ctx {
     uint32_t *d_chain = nullptr;  // chunk counters of chained tensor-core passes
     cudaEvent_t ev_full[2] = {nullptr, nullptr};  // around the full-state passes of the last run
     int64_t timed_passes = -1;
+    RunCount run;  // launches of the last run
     std::string err;
 };
 
@@ -374,6 +375,7 @@ Pass compact_pass(const Pass &p, uint64_t T) {
 // that one expansion pass writes out as the whole state.
 int run_passes(rcs_ctx *c, const Plan &plan, const uint8_t *d_ops, bool from_zero) {
     size_t first = 0;
+    RunCount count;
     std::vector<SubStage> stages;
     const int pre = from_zero ? plan_stages(plan, &stages) : 0;
     if (pre > 0) {
@@ -387,21 +389,23 @@ int run_passes(rcs_ctx *c, const Plan &plan, const uint8_t *d_ops, bool from_zer
             c->sub_cap = bytes;
         }
         int fused = 0;
-        if (run_substages(plan, stages, c->psi, c->d_sub, d_ops, c->d_err, c->stream, &fused, c->d_chain) !=
+        if (run_substages(plan, stages, c->psi, c->d_sub, d_ops, c->d_err, c->stream, &fused, c->d_chain, &count) !=
             RCS_OK)
             return fail(c, RCS_ERR_CUDA, "sub-state stages: " + take_launch_error());
         c->zero_pending = false;
         first = size_t(pre + fused);
-    } else if (int rc = materialize(c); rc != RCS_OK) {
-        return rc;
+    } else {
+        if (c->zero_pending) ++count.kernels;
+        if (int rc = materialize(c); rc != RCS_OK) return rc;
     }
     cudaEventRecord(c->ev_full[0], c->stream);
-    int64_t launches = 0;
-    if (launch_pass_range(plan, c->psi, c->n, first, plan.passes.size(), 0, d_ops, c->d_err, c->stream, &launches,
+    const int64_t before = count.passes;
+    if (launch_pass_range(plan, c->psi, c->n, first, plan.passes.size(), 0, d_ops, c->d_err, c->stream, &count,
                           c->d_chain) != RCS_OK)
         return fail(c, RCS_ERR_CUDA, "launch of a full-state pass failed: " + take_launch_error());
     cudaEventRecord(c->ev_full[1], c->stream);
-    c->timed_passes = launches;
+    c->timed_passes = count.passes - before;
+    c->run = count;
     c->sums_valid = false;
     return RCS_OK;
 }
@@ -469,7 +473,7 @@ int launch_plan_pass(void *psi, int n, const Pass &p, const uint8_t *ops, int *d
 }
 
 int run_substages(const Plan &plan, const std::vector<SubStage> &stages, void *psi, void *sub, const uint8_t *d_ops,
-                  int *d_err, void *stream, int *fused, uint32_t *chain_sync) {
+                  int *d_err, void *stream, int *fused, uint32_t *chain_sync, RunCount *count) {
     const bool tf32 = plan_tf32(plan);
     *fused = 0;
     uint8_t *buf = static_cast<uint8_t *>(sub);
@@ -491,9 +495,9 @@ int run_substages(const Plan &plan, const std::vector<SubStage> &stages, void *p
                 }
             if (launch_expand(next, m, cur, inner, stream) != RCS_OK) return RCS_ERR_CUDA;
         }
-        int64_t launches = 0;
+        ++count->kernels;
         if (launch_pass_range(plan, next, m, size_t(st.first), size_t(st.first + st.count), st.tmask, d_ops, d_err,
-                              stream, &launches, chain_sync) != RCS_OK)
+                              stream, count, chain_sync) != RCS_OK)
             return RCS_ERR_CUDA;
         cur = next;
         cur_mask = st.tmask;
@@ -503,8 +507,11 @@ int run_substages(const Plan &plan, const std::vector<SubStage> &stages, void *p
         const int rc = launch_pass_tc_from_sub(psi, plan.n, plan.passes[after], d_ops + plan.tc_offset[after], d_err,
                                                stream, tf32, cur, cur_mask);
         if (rc == RCS_OK) *fused = 1;
+        ++count->passes;
+        ++count->kernels;
         return rc;
     }
+    ++count->kernels;
     return launch_expand(psi, plan.n, cur, cur_mask, stream);
 }
 
@@ -513,7 +520,7 @@ bool plan_pairs_at(const Plan &plan, size_t i, size_t end, int n) {
 }
 
 int launch_pass_range(const Plan &plan, void *psi, int n, size_t first, size_t end, uint64_t T, const uint8_t *d_ops,
-                      int *d_err, void *stream, int64_t *launches, uint32_t *chain_sync) {
+                      int *d_err, void *stream, RunCount *count, uint32_t *chain_sync) {
     const bool tf32 = plan_tf32(plan);
     const bool images = plan.tc_offset.size() == plan.passes.size();
     // chains of passes: the split looks at targets only, so the matrices are left out
@@ -539,17 +546,19 @@ int launch_pass_range(const Plan &plan, void *psi, int n, size_t first, size_t e
     bool backwards = false;  // launches walk the state in turn from either end: L2 still holds the last part
     for (size_t i = first; i < end; backwards = !backwards) {
         if (!chain.empty() && chain[i - first] > 1) {
-            const int count = chain[i - first];
+            const int len = chain[i - first];
             const Pass *ps[8];
             const void *ops[8];
-            for (int j = 0; j < count; ++j) {
+            for (int j = 0; j < len; ++j) {
                 ps[j] = &shape[i - first + size_t(j)];
                 ops[j] = d_ops + plan.tc_offset[i + size_t(j)];
             }
-            const int rc = launch_chain_tc(psi, n, ps, ops, count, chain_sync, d_err, stream, backwards);
+            const int rc = launch_chain_tc(psi, n, ps, ops, len, chain_sync, d_err, stream, backwards);
             if (rc == RCS_OK) {
-                *launches += count;
-                i += size_t(count);
+                count->passes += len;
+                ++count->kernels;
+                ++count->chains;
+                i += size_t(len);
                 continue;
             }
             if (rc != RCS_ERR_UNSUPPORTED) return RCS_ERR_CUDA;
@@ -562,13 +571,15 @@ int launch_pass_range(const Plan &plan, void *psi, int n, size_t first, size_t e
             if (launch_pair_tc(psi, n, p, p2, d_ops + plan.pair_offset[i], d_ops + plan.pair_offset[i + 1], d_err,
                                stream) != RCS_OK)
                 return RCS_ERR_CUDA;
-            ++*launches;
+            ++count->passes;
+            ++count->kernels;
             i += 2;
             continue;
         }
         const uint8_t *ops = images && plan.tc_offset[i] >= 0 ? d_ops + plan.tc_offset[i] : nullptr;
         if (launch_plan_pass(psi, n, p, ops, d_err, stream, tf32, backwards) != RCS_OK) return RCS_ERR_CUDA;
-        ++*launches;
+        ++count->passes;
+        ++count->kernels;
         ++i;
     }
     return RCS_OK;
@@ -891,7 +902,6 @@ int rcs_apply_unitaries(rcs_ctx *c, size_t count, const int32_t *k, const int32_
         if (int rc = unitary_pass(c, k[i], targets + off, u_re_im[i], &plan.passes[i]); rc != RCS_OK) return rc;
         off += size_t(k[i]);
     }
-    if (int rc = materialize(c); rc != RCS_OK) return rc;
     std::vector<uint8_t> img;
     build_ops_images(plan, &img);
     if (!img.empty()) {
@@ -1000,6 +1010,14 @@ int rcs_last_pass_timing(rcs_ctx *c, float *ms, int64_t *full_passes) {
     RCS_CUDA(c, cudaEventSynchronize(c->ev_full[1]), "event sync");
     RCS_CUDA(c, cudaEventElapsedTime(ms, c->ev_full[0], c->ev_full[1]), "event time");
     *full_passes = c->timed_passes;
+    return RCS_OK;
+}
+
+int rcs_last_run_launches(rcs_ctx *c, int64_t *kernels, int64_t *chains) {
+    if (!c || !kernels || !chains) return fail(c, RCS_ERR_ARG, "null argument");
+    if (c->timed_passes < 0) return fail(c, RCS_ERR_ARG, "no circuit has run on this context");
+    *kernels = c->run.kernels;
+    *chains = c->run.chains;
     return RCS_OK;
 }
 

@@ -569,18 +569,18 @@ int launch_sampling(rcs_batch *b, InstHost &h, cudaStream_t st) {
 int record_chain(rcs_batch *b, InstHost &h, cudaStream_t st) {
     size_t first = 0;
     int rc = RCS_OK;
+    RunCount count;
     if (h.prefix > 0) {
         int fused = 0;
-        if ((rc = run_substages(h.plan, h.stages, h.psi, h.d_sub, h.d_ops, b->d_err, st, &fused, nullptr)) !=
+        if ((rc = run_substages(h.plan, h.stages, h.psi, h.d_sub, h.d_ops, b->d_err, st, &fused, nullptr, &count)) !=
             RCS_OK)
             return bfail(b, rc, "sub-state stages: " + take_launch_error());
         first = size_t(h.prefix + fused);
     } else if ((rc = launch_init_zero(h.psi, h.n, st)) != RCS_OK) {
         return bfail(b, rc, "reset: " + take_launch_error());
     }
-    int64_t launches = 0;
-    if ((rc = launch_pass_range(h.plan, h.psi, h.n, first, h.plan.passes.size(), 0, h.d_ops, b->d_err, st,
-                                &launches, nullptr)) != RCS_OK)
+    if ((rc = launch_pass_range(h.plan, h.psi, h.n, first, h.plan.passes.size(), 0, h.d_ops, b->d_err, st, &count,
+                                nullptr)) != RCS_OK)
         return bfail(b, rc, "pass launch: " + take_launch_error());
     return launch_sampling(b, h, st);
 }

@@ -136,6 +136,12 @@ struct SubStage {
     uint64_t tmask = 0;        // qubits of the sub-state (cumulative over the stages)
 };
 int plan_stages(const Plan &plan, std::vector<SubStage> *stages);
+// What a run launched.
+struct RunCount {
+    int64_t passes = 0;   // passes over a state (a two-unitary round trip once, each pass of a chain)
+    int64_t kernels = 0;  // kernel launches, zero fills and expansions among them
+    int64_t chains = 0;   // those of them that ran a chain of passes
+};
 // Device bytes of a stage's sub-state of m qubits (whole 256-byte lines: the passes move up to
 // 32 aligned bytes at a time), and of the buffers of the stages (one after another).
 inline size_t substate_stride(int m) { return m < 5 ? size_t(256) : size_t(8) << m; }
@@ -145,9 +151,9 @@ size_t substage_bytes(const std::vector<SubStage> &stages);
 // expansion into psi or, when the next pass can read a sub-state, that pass taking the
 // last sub-state as input (*fused = 1: the caller resumes one pass later). `sub` holds
 // substage_bytes(stages). chain_sync: scratch for chains (launch_pass_range), or null.
-// Asynchronous; launch error text kept.
+// *count: what was launched is added. Asynchronous; launch error text kept.
 int run_substages(const Plan &plan, const std::vector<SubStage> &stages, void *psi, void *sub,
-                  const uint8_t *d_ops, int *d_err, void *stream, int *fused, uint32_t *chain_sync);
+                  const uint8_t *d_ops, int *d_err, void *stream, int *fused, uint32_t *chain_sync, RunCount *count);
 // Launches one pass of a plan on a 2^n-amplitude state (ops: its operand image, if any).
 int launch_plan_pass(void *psi, int n, const Pass &p, const uint8_t *ops, int *d_err, void *stream, bool tf32,
                      bool backwards = false);
@@ -242,9 +248,9 @@ bool plan_pairs_at(const Plan &plan, size_t i, size_t end, int n);
 // Launches passes [first, end) of a plan on the 2^n-amplitude state psi, their targets
 // renumbered into the sub-state of mask T when T != 0; consecutive tensor-core passes
 // share a round trip where plan_pairs_at says so, and run as chains (tc_chain_lengths) when
-// chain_sync is given. *launches counts passes (a two-unitary round trip once).
+// chain_sync is given. *count: what was launched is added.
 int launch_pass_range(const Plan &plan, void *psi, int n, size_t first, size_t end, uint64_t T, const uint8_t *d_ops,
-                      int *d_err, void *stream, int64_t *launches, uint32_t *chain_sync);
+                      int *d_err, void *stream, RunCount *count, uint32_t *chain_sync);
 
 // Sampler / readout (k_sample.cu)
 // to_stored: caller basis index -> stored index (the state's qubit layout). Blocks are

@@ -20,24 +20,31 @@ SETS = {
 }
 
 
-@pytest.mark.parametrize("n", [24, 25])
-@pytest.mark.parametrize("kind", sorted(SETS))
-def test_chain_equals_single_passes_on_a_full_state(n, kind):
+def items_of(n, kind):
     rng = np.random.default_rng(100 + n)
-    psi = rng.standard_normal(2 << n, dtype=np.float32).view(np.complex64)
-    psi *= np.float32(2.0 ** (-(n + 1) / 2))
     items = []
     for _ in range(7):
         q, _ = np.linalg.qr(rng.standard_normal((64, 64)) + 1j * rng.standard_normal((64, 64)))
         items.append((SETS[kind](n, rng).astype(np.int32), q))
-    got = []
+    return items
+
+
+@pytest.mark.parametrize("n", [24, 25])
+@pytest.mark.parametrize("kind", sorted(SETS))
+def test_chain_equals_single_passes_on_a_full_state(n, kind):
+    psi = np.random.default_rng(n).standard_normal(2 << n, dtype=np.float32).view(np.complex64)
+    psi *= np.float32(2.0 ** (-(n + 1) / 2))
+    items = items_of(n, kind)
+    got, chains = [], []
     for calls in ([[it] for it in items], [items]):  # a call with one unitary cannot chain
         ctx = capi.rcs_create(n, capi.RCS_PREC_BF16X3)
         try:
             capi.rcs_state_write(ctx, psi)
             for c in calls:
                 capi.rcs_apply_unitaries(ctx, c)
+            chains.append(capi.rcs_last_run_launches(ctx)[1])
             got.append(capi.rcs_state_read(ctx).view(np.uint64))
         finally:
             capi.rcs_destroy(ctx)
+    assert chains[0] == 0 and chains[1] >= 3
     assert np.array_equal(*got)

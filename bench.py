@@ -593,6 +593,7 @@ def main():
             ms_p, full = capi.rcs_last_pass_timing(ctx)
             pass_ms.append(ms_p)
             timed_full = full
+            timed_launches = capi.rcs_last_run_launches(ctx)
         t_end.record(stream)
         barrier()
     total_ms = t_start.elapsed_time(t_end)
@@ -612,27 +613,22 @@ def main():
     # expansion of the last sub-state, before the timed region of the passes
     full_passes = timed_full
     t_pass_s = statistics.median(pass_ms) / 1e3 / full_passes
-    # launches per step: sub-state reset, expansions between sub-states, the final expansion
-    # unless the first full pass reads the last sub-state, every pass, block sums, the 3-phase
-    # scan, the sampler (locate, 3-phase scan of its per-block counts, order, resolve) and the
-    # 2-phase XEB
-    stages = int(info["prefix_stages"])
-    fused = prefix > 0 and full_passes == passes - prefix - 1
-    setup = 1 + max(stages - 1, 0) + (0 if (prefix == 0 or fused) else 1)
-    # BF16x3 passes on 24 or more qubits run chained, two or three in one launch: count three
-    chained = args.precision == "bf16x3" and not pairs and n >= 24
-    gpu_launches = (-(-(passes - pairs) // 3) if chained else passes - pairs) + setup + 1 + 3 + 6 + 2
-    bytes_per_launch = 16.0 * 2.0**n  # of one pass; chained passes share one trip through HBM
-    achieved = bytes_per_launch / t_pass_s / 1e9
-    # traffic: DRAM bytes per launch from an ncu capture of the same kernel (None for a kernel
+    # launches of a step: the run's own, as the library counts them, block sums, the 3-phase scan,
+    # the sampler (locate, 3-phase scan of its per-block counts, order, resolve) and the 2-phase XEB
+    run_kernels, chains = timed_launches
+    gpu_launches = (run_kernels + 1 + 3 + 6 + 2) * args.steps
+    chained = chains > 0
+    bytes_per_pass = 16.0 * 2.0**n  # chained passes share one trip through HBM
+    achieved = bytes_per_pass / t_pass_s / 1e9
+    # traffic: DRAM bytes per pass from an ncu capture of the same kernel (None for a kernel
     # not captured since it last changed)
     traffic = PAIR_DRAM_BYTES_PER_AMP if pairs else TC_DRAM_BYTES_PER_AMP[args.precision]
     roofline = {"bound": "hbm", "achieved": achieved, "peak": peaks["hbm_gbs"], "unit": "GB/s",
                 "frac": achieved / peaks["hbm_gbs"], "traffic": traffic * 2.0**n if traffic else None,
                 "traffic_src": "ncu capture at 27 qubits scaled by 2^(n-27)" if traffic else None,
                 "kernel": "k_pair_tc (two unitaries per launch)" if pairs else "k_fused_tc", "peak_src": peaks["src"],
-                "algorithmic_bytes_per_launch": bytes_per_launch, "launches_per_step": full_passes,
-                "mean_launch_ms": t_pass_s * 1e3}
+                "algorithmic_bytes_per_pass": bytes_per_pass, "passes_per_step": full_passes,
+                "mean_pass_ms": t_pass_s * 1e3}
     if chained:
         # per pass, as if each made its own trip: above 1 because two or three share one through L2
         # (HBM itself moves 1/2 to 1/3 of these bytes; the SM's tile pipeline is the bound)

@@ -631,6 +631,19 @@ int launch_pass_plain(void *psi, int n, const Pass &p, void *stream) {
     return check_launch();
 }
 
+// Dynamic shared memory of a fused pass's launch whose kernel needs `smem`: so much that no SM
+// takes more than its even share of the CTAs. They come in (launch_after) while those of the
+// passes before sit on most SMs; without this they crowded onto the others, as many to an SM as
+// fit, and the pass took as much longer. Back to back on 19 qubits, us a pass: width 5 (128
+// CTAs) 9.6 to 20.2 (by its targets), now 5.7 to 9.9; width 6 (128) 13.5 to 20.2, now 8.5 to
+// 12.1; width 3 (256) 4.5 to 4.8, now 3.6 to 3.7. On 20 qubits width 5 (256) 11.8 to 24.6, now
+// 8.9 to 16.5. Without overlap with the pass before: 8.5 to 12.7, 10.7 to 14.7, 6.4, 10.7 to 18.8.
+constexpr size_t kSmemPerSm = 228 * 1024;  // each CTA takes 1 KB of it for the system
+static size_t spread_smem(size_t smem, unsigned grid) {
+    const unsigned sms = unsigned(device_sm_count()), share = (grid + sms - 1) / sms;
+    return std::max(smem, kSmemPerSm / (share + 1));
+}
+
 // Shared-memory attribute of k_fused_simt<K> on the current device (once).
 template <int K>
 static int simt_attr() {
@@ -639,7 +652,7 @@ static int simt_attr() {
     cudaGetDevice(&dev);
     if (dev >= 0 && dev < 64 && attr_done[dev]) return RCS_OK;
     const cudaError_t e = cudaFuncSetAttribute(k_fused_simt<K>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                               int(8 * kSimtSlots * simt_unit_bytes<K>()));
+                                               int(std::max(kSmemPerSm / 2, size_t(8 * kSimtSlots * simt_unit_bytes<K>()))));
     if (e != cudaSuccess) return note_launch_error("fused kernel shared-memory attribute", e);
     if (dev >= 0 && dev < 64) attr_done[dev] = true;
     return RCS_OK;
@@ -653,7 +666,8 @@ static int wide_attr() {
     cudaGetDevice(&dev);
     if (dev >= 0 && dev < 64 && attr_done[dev]) return RCS_OK;
     const cudaError_t e =
-        cudaFuncSetAttribute(k_fused_wide<K>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(wide_smem_bytes<K>()));
+        cudaFuncSetAttribute(k_fused_wide<K>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             int(std::max(kSmemPerSm / 2, wide_smem_bytes<K>())));
     if (e != cudaSuccess) return note_launch_error("wide fused kernel shared-memory attribute", e);
     if (dev >= 0 && dev < 64) attr_done[dev] = true;
     return RCS_OK;
@@ -721,7 +735,8 @@ static int launch_simt_k(float2 *psi, int n, const Pass &p, bool backwards, cuda
     if (int rc = simt_attr<K>(); rc != RCS_OK) return rc;
     // persistent: the resident CTAs, never more than the units need
     const unsigned grid = grid_for(a.units, 8, device_sm_count(), simt_blocks_per_sm<K>());
-    const cudaError_t e = launch_after(k_fused_simt<K>, grid, 256, 8 * kSimtSlots * simt_unit_bytes<K>(), st, psi, a);
+    const size_t smem = spread_smem(8 * kSimtSlots * simt_unit_bytes<K>(), grid);
+    const cudaError_t e = launch_after(k_fused_simt<K>, grid, 256, smem, st, psi, a);
     return e == cudaSuccess ? RCS_OK : note_launch_error("fused pass", e);
 }
 
@@ -736,7 +751,8 @@ static int launch_wide_k(float2 *psi, int n, const Pass &p, const uint8_t *ops, 
     const uint64_t tiles = (a.slices + WideShape<K>::T - 1) / WideShape<K>::T;
     const uint64_t resident = uint64_t(device_sm_count()) * wide_blocks_per_sm<K>();
     const unsigned grid = unsigned(tiles < resident ? tiles : resident);
-    const cudaError_t e = launch_after(k_fused_wide<K>, grid, kWideThreads, wide_smem_bytes<K>(), st, psi,
+    const size_t smem = spread_smem(wide_smem_bytes<K>(), grid);
+    const cudaError_t e = launch_after(k_fused_wide<K>, grid, kWideThreads, smem, st, psi,
                                        reinterpret_cast<const float2 *>(ops), a);
     return e == cudaSuccess ? RCS_OK : note_launch_error("wide fused pass", e);
 }

@@ -17,6 +17,7 @@ struct Launch {
     std::string kernel;
     unsigned grid;
     int device;
+    size_t smem;
 };
 
 int g_device = 0;
@@ -51,7 +52,7 @@ cudaError_t note(cudaError_t e) {
     return e;
 }
 
-cudaError_t launch(const void *fun, dim3 grid) {
+cudaError_t launch(const void *fun, dim3 grid, size_t smem) {
     const std::string name = kernels().count(fun) ? kernels()[fun] : "?";
     if (g_fail_times > 0 && name.find(g_fail_kernel) != std::string::npos) {
         if (g_fail_skip > 0) {
@@ -61,7 +62,7 @@ cudaError_t launch(const void *fun, dim3 grid) {
             return note(g_fail_code);
         }
     }
-    g_launches.push_back({name, grid.x, g_device});
+    g_launches.push_back({name, grid.x, g_device, smem});
     return cudaSuccess;
 }
 
@@ -96,6 +97,7 @@ int fake_launches() { return int(g_launches.size()); }
 const char *fake_launch_kernel(int i) { return g_launches[size_t(i)].kernel.c_str(); }
 int fake_launch_device(int i) { return g_launches[size_t(i)].device; }
 int fake_launch_grid(int i) { return int(g_launches[size_t(i)].grid); }
+int fake_launch_smem(int i) { return int(g_launches[size_t(i)].smem); }
 
 // ---- registration and launches
 void **__cudaRegisterFatBinary(void *) {
@@ -128,8 +130,12 @@ cudaError_t __cudaGetKernel(cudaKernel_t *k, const void *fun) {
     *k = reinterpret_cast<cudaKernel_t>(const_cast<void *>(fun));
     return cudaSuccess;
 }
-cudaError_t __cudaLaunchKernel(cudaKernel_t k, dim3 grid, dim3, void **, size_t, cudaStream_t) { return launch(k, grid); }
-cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t *c, const void *fun, void **) { return launch(fun, c->gridDim); }
+cudaError_t __cudaLaunchKernel(cudaKernel_t k, dim3 grid, dim3, void **, size_t smem, cudaStream_t) {
+    return launch(k, grid, smem);
+}
+cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t *c, const void *fun, void **) {
+    return launch(fun, c->gridDim, c->dynamicSmemBytes);
+}
 
 // ---- errors and devices
 cudaError_t cudaGetLastError() {

@@ -160,6 +160,7 @@ struct SimtArgs {
     uint64_t coff[1 << (K - 1)];  // copy c of a unit (see k_fused_simt)
     uint64_t units;
     uint32_t depth;               // units in a warp's ring, 2..kSimtSlots
+    uint32_t step;                // width 4: the CTA's warps start each unit together
     uint32_t flip;                // XORed into the unit numbers: 0, or units - 1 to walk the state backwards
     int t[K];                     // ascending
     int8_t rpos[5];               // index bit of lane (slice) bit i: the 5 lowest non-target qubits
@@ -186,11 +187,20 @@ template <int K>
 uint32_t simt_depth(int lowest) {
     return K == 3 || (K == 4 && lowest < 5) ? 2u : 3u;
 }
+// Whether the warps of a CTA start each unit together at width 4, where multiplying a unit takes
+// a warp nearly as long as HBM takes to serve it. Left alone they drift apart, and in a large
+// state the copies of neighbouring units no longer come together: ms a pass at 32 qubits, alone
+// and in step, targets on the top bits 11.9-12.1 and 11.2, in the middle 11.6-11.7 and 10.7,
+// spread from bit 0 up 11.6 and 10.8 (one slice per thread, 8-byte copies: 11.4, 11.0, 11.2); at
+// 28 qubits 698-710 and 678 us, 669-715 and 678, 708 and 664. At 27 they take 340 and 343, 333
+// and 342, and below that it is slower as well. With the lowest target on bits 1 to 4, or on
+// bits 0 and 1 together, it costs 5 to 25% at every size.
+bool simt_in_step(int n, int lowest, bool quad) { return n >= 28 && (lowest >= 5 || (lowest == 0 && !quad)); }
 
 // A warp applies U to a unit of 32 neighbouring slices, one per lane, persistent over the
 // units (grid-stride). Units come through a ring of shared-memory slots of the warp's own, so
 // the copies of the next ones are in flight while it multiplies, and no block barrier is
-// needed. Copies are 16 bytes wide and bypass L1: for each pair of amplitudes (j = 2 c,
+// needed (simt_in_step says where there is one all the same). Copies are 16 bytes wide and bypass L1: for each pair of amplitudes (j = 2 c,
 // 2 c + 1, which differ in the lowest target) the unit's 64 values are one 512-byte block in
 // the order of their index bits: bit tb is the lowest target (bit 5 if that lies above bit 4),
 // the others are the lane bits. So the lanes of a copy go up both in memory and in the slot.
@@ -260,15 +270,19 @@ __global__ void __launch_bounds__(256, simt_blocks_per_sm<K>())
         asm volatile("st.global.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(p), "f"(x.x), "f"(x.y), "f"(y.x), "f"(y.y)
                      : "memory");
     };
-    uint32_t u = blockIdx.x * 8u + (threadIdx.x >> 5);
+    const uint32_t first = blockIdx.x * 8u;
+    uint32_t u = first + (threadIdx.x >> 5);
     const bool deep = a.depth == 3;
+    const bool step = K == 4 && a.step;
     grid_wait();  // the pass before (launch_after)
     issue(u, 0);
     if (deep) issue(u + warps, 1);
     uint32_t slot = 0, fill = deep ? 2 : 1;
 #pragma unroll 1
-    for (; u < a.units; u += warps) {
-        __syncwarp();  // every lane has read the slot that is filled next
+    for (uint32_t c = first; c < a.units; c += warps, u += warps) {  // as many trips for every warp of the CTA
+        if (step) __syncthreads();
+        else __syncwarp();  // every lane has read the slot that is filled next
+        if (u >= a.units) continue;  // fewer than 8 units
         issue(u + (deep ? 2 : 1) * warps, fill);
         if (++fill == a.depth) fill = 0;
         if (deep) asm volatile("cp.async.wait_group 2;" ::: "memory");  // this unit's copies
@@ -731,7 +745,8 @@ static int launch_simt_k(float2 *psi, int n, const Pass &p, bool backwards, cuda
         a.coff[c] = quad ? ((c & 1) ? 8ull << a.rpos[4] : 0ull) + a.joff[4 * (c >> 1)] : a.joff[2 * c];
     a.units = 1ull << (n - K - 5);
     a.flip = backwards ? uint32_t(a.units - 1) : 0u;
-    a.depth = simt_depth<K>(p.t[0]);
+    a.step = K == 4 && simt_in_step(n, p.t[0], quad);
+    a.depth = a.step ? 2u : simt_depth<K>(p.t[0]);
     if (int rc = simt_attr<K>(); rc != RCS_OK) return rc;
     // persistent: the resident CTAs, never more than the units need
     const unsigned grid = grid_for(a.units, 8, device_sm_count(), simt_blocks_per_sm<K>());

@@ -178,7 +178,7 @@ int rcs_reset(rcs_ctx *ctx);
  * (such passes cannot stream memory at full rate). This is invisible to the caller:
  * samples, amplitudes and XEB use the circuit's own qubit numbering, later circuits
  * follow the layout, and rcs_state_read/write/device first restore the identity
- * layout (at most five exact swap passes). rcs_qubit_layout reports it. */
+ * layout (one exact permutation pass). rcs_qubit_layout reports it. */
 int rcs_apply_circuit(rcs_ctx *ctx, const rcs_gate *gates, size_t n_gates);
 
 /* Applies one dense k-qubit unitary (1 <= k <= 7) to targets[0..k-1] (distinct,
@@ -270,7 +270,7 @@ int rcs_state_device(rcs_ctx *ctx, void **d_state);
  * RCS_ERR_ARG for an out-of-range bitstring or an unusable state), then clears them. */
 int rcs_sync(rcs_ctx *ctx);
 
-/* Test hook for the bounded waits of the tensor-core kernels (single passes and pair
+/* Test hook for the bounded waits of the tensor-core kernels (single, chained and pair
  * passes), process-wide: while skip_tile >= 0, every tensor-core launch has its first CTA
  * skip the MMAs of its tile number skip_tile (it issues and commits nothing for that
  * tile), so the waits for that tile run out after wait_limit_s seconds of SM clock; the

@@ -2,15 +2,19 @@
 // state, and the copy of a caller-order range out of a permuted one.
 //
 // k_permute: psi[x] <- psi[m(x)], where m moves index bits. A tile is the set of
-// amplitudes that differ only in the bits B = (moved bits and the lowest others, 12 in
-// all): m maps each tile to itself, so a CTA reads a tile into shared memory, and writes
-// it back in the new order: one read and one write of the state however many bits move
-// (bound by HBM: 16 * 2^n bytes). Bits 0 and up to 4 neighbours are in B, so global loads
-// and stores are 16 bytes wide in runs of at least 2^5 amplitudes. The shared index is
-// XOR-swizzled (its bits 4.. folded onto bits 0..3), which spreads reads along any moved
-// bits over the banks. The exchange of circuit qubits with the lowest bits that a planned
-// layout needs (up to 5 swaps) used to run as one k_plain_2q pass per swap: 1.35 ms for 4
-// swaps at 27 qubits.
+// amplitudes that differ only in the bits B = (bit 0, the moved bits and the lowest others,
+// 12 in all): m maps each tile to itself, so a CTA reads a tile into shared memory, and
+// writes it back in the new order: one read and one write of the state however many bits
+// move. Bit 0 is in B, so global loads and stores are 16 bytes wide. The layouts that the
+// planner chooses swap up to 5 low bits with high ones, so bits 1..4 are in B too and runs
+// are at least 2^5 amplitudes; a loaded file may move 11 high bits in a pass, whose runs are
+// then 2 amplitudes, half a sector. The shared index is XOR-swizzled (its bits 4..7 and
+// 8..11 folded onto bits 0..3), which keeps reads along bits that differ mod 4 on different
+// banks. Measured (a planned layout, 3 swaps): 8.1 us at 19 qubits, 555 us at 27,
+// where one trip through HBM takes 321: the eight float4 that a thread holds do not fit the
+// 40 registers of six CTAs per SM, and spill (DRAM 2.7 GB instead of 2.1; shared-memory
+// pipe 51% busy). The exchange of circuit qubits with the lowest bits used to run as one
+// k_plain_2q pass per swap: 1.35 ms for 4 swaps at 27 qubits.
 #include <algorithm>
 #include <bit>
 

@@ -113,7 +113,7 @@ __device__ __forceinline__ uint32_t swz(uint32_t c) { return c ^ ((c >> 6) & 15u
 // targets and the lowest qubits, so every pass maps a chunk to itself. CTA b works on pass
 // b mod npass; the CTAs of a pass take its tiles in chunk order, and a pass starts a chunk
 // once the pass before it has stored all of it. A chunk then still sits in L2: with chunks
-// of 8 or 16 MB and a window of 64 to 80 MB between passes, the first pass reads HBM, the
+// of 8 MB and a window of 64 or 80 MB between passes, the first pass reads HBM, the
 // last one's stores go back to it, and all else runs at L2's rate: at 27 qubits a pair of
 // passes takes 458 us against 2 x 323 one after the other (where HBM runs at its peak), and
 // the SM's own pipeline (2.1 us per tile: 1.5 without any copies and stores) is the bound.
@@ -1124,9 +1124,13 @@ static int launch_tc(void *psi, int n, const Pass &p, const void *d_ops, int *d_
     // the memory-order and sub-state loaders walk forwards
     const bool staged = low_targets(p) >= 4;
     a.flip = backwards && !staged && !sub ? a.tiles - 1 : 0;
-    // A state beyond L2 streams best with one tile (two units) in flight per SM: with all five
-    // units HBM serves the same bytes more slowly (328 against 351 us a BF16x3 pass at 27 qubits;
-    // from L2 five units are faster, 23.4 against 24.7 us at 23). TF32x3 times alike with 2 to 4.
+    // A state beyond L2 streams best with one tile (two units) in flight per SM: with more HBM serves
+    // the same bytes more slowly (a BF16x3 pass at 27 qubits with 2 / 3 / 4 units 325-333 / 347-353
+    // / 351-359 us; from L2 five are faster, 23.4 against 24.7 us at 23). With two a single pass on 28
+    // to 31 qubits is still up to 3% slower than with 8-byte copies through L1 (644-656 against
+    // 631-647 us at 28), at 27 as fast; most passes run chained. TF32x3 keeps four at every size: up
+    // to 24 qubits they are the faster (55-57 against 57-58 us at 24), beyond that two would be
+    // (332-335 against 359-372 us at 27).
     a.depth = !tf32 && (8ull << n) > (uint64_t(64) << 20) ? 2u : uint32_t(tf32 ? Layout<true>::kSlots : Layout<false>::kSlots);
     // qubits varying inside a tile: the targets plus the 7 lowest other qubits
     const uint64_t V = tile_qubits(p, n);
@@ -1172,19 +1176,20 @@ int launch_pass_tc_from_sub(void *psi, int n, const Pass &p, const void *d_ops, 
 // ---------------------------------------------------------------- chains of passes
 
 // The chunk of a chain of `count` passes: every tile's qubits of every pass, filled up with
-// the lowest other qubits to at least kChunkMinLog2. 0 if the passes cannot form a chain.
+// the lowest other qubits to kChunkLog2. 0 if the passes cannot form a chain.
 static uint64_t chain_chunk(const Pass *const *p, int count, int n) {
     uint64_t C = 0;
     for (int i = 0; i < count; ++i) {
         if (p[i]->kind != PASS_TC || p[i]->k != tc::K || low_targets(*p[i]) >= 4) return 0;
         C |= tile_qubits(*p[i], n);
     }
-    for (int qb = 0; qb < n && std::popcount(C) < tc::kChunkMinLog2; ++qb) C |= 1ull << qb;
+    if (std::popcount(C) > tc::kChunkLog2) return 0;
+    for (int qb = 0; qb < n && std::popcount(C) < tc::kChunkLog2; ++qb) C |= 1ull << qb;
     return C;
 }
 
 size_t tc_chain_sync_bytes(int n) {
-    return n < tc::kChainMinQubits ? 0 : (1 + (size_t(tc::kChainMax) << (n - tc::kChunkMinLog2))) * sizeof(uint32_t);
+    return n < tc::kChainMinQubits ? 0 : (1 + (size_t(tc::kChainMax) << (n - tc::kChunkLog2))) * sizeof(uint32_t);
 }
 
 std::vector<int> tc_chain_lengths(const std::vector<Pass> &passes, int n, bool tf32) {
@@ -1198,8 +1203,7 @@ std::vector<int> tc_chain_lengths(const std::vector<Pass> &passes, int n, bool t
         const Pass *p[tc::kChainMax];
         for (int c = 1; c <= tc::kChainMax && i + size_t(c) <= m; ++c) {
             p[c - 1] = &passes[i + size_t(c) - 1];
-            const uint64_t C = chain_chunk(p, c, n);
-            if (c > 1 && (C == 0 || std::popcount(C) > tc::kChunkMaxLog2[c])) break;
+            if (c > 1 && chain_chunk(p, c, n) == 0) break;
             const double cost = tc::kChainCost[c] + best[i + size_t(c)];
             if (cost < best[i]) {
                 best[i] = cost;
@@ -1225,8 +1229,8 @@ int launch_chain_tc(void *psi, int n, const Pass *const *p, const void *const *d
     tc_test_fault(&a.wait_cycles, &a.skip_tile);
     a.tiles = uint32_t((1ull << (n - K)) / M);
     a.npass = count;
-    a.clog = std::popcount(C) - K - 7;
-    a.window = uint32_t(kChainWindowBytes[count] >> (std::popcount(C) + 3));
+    a.clog = kChunkLog2 - K - 7;
+    a.window = uint32_t(kChainWindowBytes[count] >> (kChunkLog2 + 3));
     a.sync = sync;
     a.flip = backwards ? a.tiles - 1 : 0;
     a.depth = uint32_t(Layout<false>::kSlots);

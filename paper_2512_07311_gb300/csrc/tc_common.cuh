@@ -27,12 +27,12 @@ constexpr int kChainThreads = kThreads + 64;    // two more warps order the chun
 // From 128 MB a state no longer stays in L2 from one pass to the next (two passes at 24 qubits:
 // 87 us as a chain, 95 one after the other; at 23 qubits 57 against 47).
 constexpr int kChainMinQubits = 24;
-// A chunk of 8 MB gives the CTAs of a pass one or two tiles each. The larger it is, the fewer of
-// them fit the window below; two passes need chunks of up to 2^19 amplitudes, three mostly 2^19
-// to 2^21. Measured with chunks of at least 2^18 / 2^19 / 2^20 / 2^21: the 30-qubit, 14-cycle
-// circuit 35.6 / 32.9 / 32.1 / 32.9 ms, the 27-qubit, 20-cycle one 5.72 / 5.23 / 5.19 / 5.31.
-constexpr int kChunkMinLog2 = 20;
-constexpr int kChunkMaxLog2[kChainMax + 1] = {0, 0, 21, 20};
+// Amplitudes of a chunk: 8 MB, 128 tiles, one to three for each CTA of a pass. Every two passes fit
+// one (their targets and seven lowest other qubits are at most 19), three do where they share
+// enough. The larger a chunk, the fewer of them fit the window below. Measured with chunks of at
+// least 2^18 / 2^19 / 2^20 / 2^21: the 30-qubit, 14-cycle circuit 35.6 / 32.9 / 32.1 / 32.9 ms,
+// the 27-qubit, 20-cycle one 5.72 / 5.23 / 5.19 / 5.31.
+constexpr int kChunkLog2 = 20;
 // Distance between two passes of a chain. The tiles in flight in both (about 4 per SM each) and
 // the counters' round trip take some 70 MB; beyond about 80 MB for a pair and 64 MB a step for
 // three the chunks start to fall out of L2. Measured at 27 qubits, us a pass: pairs with 40 /

@@ -660,11 +660,18 @@ __global__ void __launch_bounds__(kChain ? tc::kChainThreads : tc::kThreads, 1)
         // (the even lane j, the odd lane j+1). Either way a store instruction covers 512
         // contiguous bytes (with one target below bit 6); above bit 4, 8-byte stores already
         // fill whole lines.
-        const int smode = t[0] == 0 ? (t[1] == 1 ? 3 : 1) : (t[0] < 5 ? 2 : 0);
+        //
+        // With the sub-state input most of a tile's time is this loop (the loaders copy a part of a
+        // tile only), and it is faster with the slice's base from index arithmetic, the offsets from
+        // shared memory, and 16-byte stores for the lowest target on bits 0 and 1 only: with the
+        // addresses and stores of the other passes a 30-qubit one took 2.19 to 2.29 ms (BF16x3) and
+        // 2.80 to 2.90 (TF32x3), so 2.09 and 2.29, a 27-qubit one 274 and 342 us, so 257 and 292.
+        const int smode = t[0] == 0 ? (!kSub && t[1] == 1 ? 3 : 1) : (t[0] < (kSub ? 2 : 5) ? 2 : 0);
         const bool odd = lane & 1;
         // on bits 1..4 the lane's row is the even slice of its pair, and odd lanes start at j + 1
-        const uint64_t ebase = row_bytes(smode == 2 ? srow & ~1 : srow) + (h ? ps.joff5 : 0ull) +
-                               (smode == 2 && odd ? ps.joff[1] : 0ull);
+        const uint64_t ebase = kSub ? 0ull
+                                    : row_bytes(smode == 2 ? srow & ~1 : srow) + (h ? ps.joff5 : 0ull) +
+                                          (smode == 2 && odd ? ps.joff[1] : 0ull);
         // Chain: what the last pass stores is not read again, so it leaves L2 first, and the chunks
         // that wait for their next pass stay (without it a window of 96 MB overflows L2: 281 against
         // 248 us a pass at 27 qubits).
@@ -705,7 +712,22 @@ __global__ void __launch_bounds__(kChain ? tc::kChainThreads : tc::kThreads, 1)
             const int b = i & 1;
             if (!warp_wait<!kTf32>(bar_done(b), (i >> 1) & 1, abort_flag, lim)) break;
             tc_fence_after();
-            uint8_t *dst = reinterpret_cast<uint8_t *>(a.psi) + (ebase | tile_bytes((cta + i * ctas) ^ a.flip));
+            const uint32_t tile = cta + i * ctas;
+            uint8_t *dst = nullptr;
+            uint64_t sbase = 0;  // kSub
+            if constexpr (kSub) {
+                sbase = slice_base(uint64_t(tile) * M + srow, t);
+                if (smode == 2) sbase &= ~1ull;  // the even slice of the lane pair
+            } else {
+                dst = reinterpret_cast<uint8_t *>(a.psi) + (ebase | tile_bytes(tile ^ a.flip));
+            }
+            // where local amplitude j of this warp's half goes (smode 2: j + 1 for odd lanes)
+            auto at = [&](int j) {
+                if constexpr (kSub)
+                    return reinterpret_cast<uint8_t *>(a.psi + (sbase | off[32 * h + j + (smode == 2 && odd ? 1 : 0)]));
+                else
+                    return dst + ps.joff[j];
+            };
             const uint32_t dbase = dcol_of(b) + (uint32_t(32 * q) << 16);
 #pragma unroll
             for (int c = 0; c < 2; ++c) {
@@ -714,10 +736,10 @@ __global__ void __launch_bounds__(kChain ? tc::kChainThreads : tc::kThreads, 1)
                 if (smode == 3) {
 #pragma unroll
                     for (int jj = 0; jj < 16; jj += 4)
-                        st32(dst + ps.joff[16 * c + jj], v[jj], v[jj + 1], v[jj + 2], v[jj + 3]);
+                        st32(at(16 * c + jj), v[jj], v[jj + 1], v[jj + 2], v[jj + 3]);
                 } else if (smode == 1) {
 #pragma unroll
-                    for (int jj = 0; jj < 16; jj += 2) st16(dst + ps.joff[16 * c + jj], v[jj], v[jj + 1]);
+                    for (int jj = 0; jj < 16; jj += 2) st16(at(16 * c + jj), v[jj], v[jj + 1]);
                 } else if (smode == 2) {
 #pragma unroll
                     for (int jj = 0; jj < 16; jj += 2) {
@@ -726,11 +748,11 @@ __global__ void __launch_bounds__(kChain ? tc::kChainThreads : tc::kThreads, 1)
                         const float2 recv = make_float2(__shfl_xor_sync(0xffffffffu, send.x, 1),
                                                         __shfl_xor_sync(0xffffffffu, send.y, 1));
                         const float2 x = odd ? recv : v[jj], y = odd ? v[jj + 1] : recv;
-                        st16(dst + ps.joff[16 * c + jj], x, y);
+                        st16(at(16 * c + jj), x, y);
                     }
                 } else {
 #pragma unroll
-                    for (int jj = 0; jj < 16; ++jj) st8(dst + ps.joff[16 * c + jj], v[jj]);
+                    for (int jj = 0; jj < 16; ++jj) st8(at(16 * c + jj), v[jj]);
                 }
             }
             tc_fence_before();

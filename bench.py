@@ -29,10 +29,10 @@ sys.path.insert(0, ROOT)
 from paper_2512_07311_gb300 import circuits as C  # noqa: E402
 
 METRIC = "34q 20-cycle circuit time (s), shots/s; fused-TC vs plain FP32 at 1e-5 infid"
-# DRAM bytes (read + write) per amplitude per tensor-core pass, where an ncu capture of the current
-# kernel has them (None: not captured since it last changed; the chained BF16x3 passes are in
-# profiles/k_fused_tc_chain_27q.md)
-TC_DRAM_BYTES_PER_AMP = {"bf16x3": None, "tf32x3": None}
+# DRAM bytes (read + write) per amplitude per single tensor-core pass, from ncu captures of a 2^27-amplitude
+# state (profiles/k_fused_tc_single_27q.md; chained BF16x3 passes, profiles/k_fused_tc_chain_27q.md,
+# move less and report none)
+TC_DRAM_BYTES_PER_AMP = {"bf16x3": 2.086e9 / 2**27, "tf32x3": 2.0866e9 / 2**27}
 PAIR_DRAM_BYTES_PER_AMP = (1.074e9 + 1.012e9) / 2**27  # the two-unitary kernel, captured at 27 qubits
 # the persistent batch kernel on the 64-circuit workload: DRAM bytes of one launch (ncu)
 BATCH64_TC_DRAM_BYTES = 86.469e9 + 92.177e9

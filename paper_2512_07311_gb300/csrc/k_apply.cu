@@ -192,9 +192,10 @@ uint32_t simt_depth(int lowest) {
 // state the copies of neighbouring units no longer come together: ms a pass at 32 qubits, alone
 // and in step, targets on the top bits 11.9-12.1 and 11.2, in the middle 11.6-11.7 and 10.7,
 // spread from bit 0 up 11.6 and 10.8 (one slice per thread, 8-byte copies: 11.4, 11.0, 11.2); at
-// 28 qubits 698-710 and 678 us, 669-715 and 678, 708 and 664. At 27 they take 340 and 343, 333
-// and 342, and below that it is slower as well. With the lowest target on bits 1 to 4, or on
-// bits 0 and 1 together, it costs 5 to 25% at every size.
+// 28 qubits 698-710 and 678 us, 669-715 and 678, 708 and 664. At 27 the first two take 340 and
+// 343, 333 and 342 us (the third 354 and 335), and at 25 and 26 they are slower in step as well.
+// With the lowest target on bits 1 to 4 it costs 4 to 6% from 24 qubits on, and with targets on
+// bits 0 and 1 together 15 to 25%.
 bool simt_in_step(int n, int lowest, bool quad) { return n >= 28 && (lowest >= 5 || (lowest == 0 && !quad)); }
 
 // A warp applies U to a unit of 32 neighbouring slices, one per lane, persistent over the

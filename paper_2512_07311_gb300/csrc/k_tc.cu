@@ -664,8 +664,9 @@ __global__ void __launch_bounds__(kChain ? tc::kChainThreads : tc::kThreads, 1)
         // With the sub-state input most of a tile's time is this loop (the loaders copy a part of a
         // tile only), and it is faster with the slice's base from index arithmetic, the offsets from
         // shared memory, and 16-byte stores for the lowest target on bits 0 and 1 only: with the
-        // addresses and stores of the other passes a 30-qubit one took 2.19 to 2.29 ms (BF16x3) and
-        // 2.80 to 2.90 (TF32x3), so 2.09 and 2.29, a 27-qubit one 274 and 342 us, so 257 and 292.
+        // addresses and stores of the other passes a 30-qubit one took 2.11 to 2.29 ms (BF16x3) and
+        // 2.80 to 2.90 (TF32x3), so 2.09 to 2.15 and 2.29 to 2.44, a 27-qubit one 274 and 342 us, so
+        // 257 to 261 and 292 to 299.
         const int smode = t[0] == 0 ? (!kSub && t[1] == 1 ? 3 : 1) : (t[0] < (kSub ? 2 : 5) ? 2 : 0);
         const bool odd = lane & 1;
         // on bits 1..4 the lane's row is the even slice of its pair, and odd lanes start at j + 1

@@ -86,6 +86,7 @@ struct TcArgs {
     int skip_tile;          // test hook: CTA 0 issues no MMAs for its tile skip_tile (-1: none)
     uint32_t flip;          // XORed into the tile numbers: 0, or tiles - 1 to walk the state backwards
     uint32_t depth;         // slice order: units a loader warp keeps in flight or in conversion, 2..kSlots
+    uint32_t step;          // slice order, BF16, no chain: the CTA's loader warps start each unit together
     // Chain (kChain): see the comment at k_fused_tc.
     int npass;              // passes of the chain, 2..kChainMax
     int clog;               // log2 of the tiles in a chunk
@@ -144,6 +145,7 @@ __global__ void __launch_bounds__(kChain ? tc::kChainThreads : tc::kThreads, 1)
     auto bar_done = [&](int b) { return bar0 + 16u + 8u * uint32_t(b); };
     auto bar_free = [&](int b) { return bar0 + 32u + 8u * uint32_t(b); };
     auto bar_loaded = [&](int b) { return bar0 + 48u + 8u * uint32_t(b); };    // stage b holds the tile's inputs
+    const uint32_t bar_step = bar0 + 48u;  // slice order: the loader warps reached the unit (a.step)
     auto bar_outready = [&](int b) { return bar0 + 64u + 8u * uint32_t(b); };  // stage b holds the tile's outputs
     auto bar_sfree = [&](int b) { return bar0 + 80u + 8u * uint32_t(b); };     // stage b read out by the stores
     // TF32: A is filled and consumed in two K halves (inputs 0..31 by loader warps 0-3,
@@ -238,7 +240,7 @@ __global__ void __launch_bounds__(kChain ? tc::kChainThreads : tc::kThreads, 1)
                 mbar_init(bar_done_a(b), 1);
                 mbar_init(bar_done(b), 1);
                 mbar_init(bar_free(b), kEpiWarps);
-                mbar_init(bar_loaded(b), kLoaderWarps * 32);
+                mbar_init(bar_loaded(b), kStaged ? kLoaderWarps * 32 : kLoaderWarps);
                 mbar_init(bar_outready(b), kEpiWarps);
                 mbar_init(bar_sfree(b), kEpiWarps);
             }
@@ -556,6 +558,12 @@ __global__ void __launch_bounds__(kChain ? tc::kChainThreads : tc::kThreads, 1)
                 for (int ch = 0; ch < 2; ++ch) {
                     const uint32_t u = 2 * i + uint32_t(ch);
                     __syncwarp();  // every lane has read the slot that is filled next
+                    if constexpr (!kTf32 && !kChain) {
+                        if (a.step) {
+                            if (lane == 0) mbar_arrive(bar_step);
+                            if (!(ok = warp_wait<!kTf32>(bar_step, u & 1u, abort_flag, lim))) break;
+                        }
+                    }
                     if (!(ok = top_up(u))) break;
                     const uint32_t later = issued - u - 1;  // units in flight behind this one
                     if (later >= kSlots - 1) asm volatile("cp.async.wait_group %0;" ::"n"(kSlots - 1) : "memory");
@@ -1149,12 +1157,16 @@ static int launch_tc(void *psi, int n, const Pass &p, const void *d_ops, int *d_
     a.flip = backwards && !staged && !sub ? a.tiles - 1 : 0;
     // A state beyond L2 streams best with one tile (two units) in flight per SM: with more HBM serves
     // the same bytes more slowly (a BF16x3 pass at 27 qubits with 2 / 3 / 4 units 325-333 / 347-353
-    // / 351-359 us; from L2 five are faster, 23.4 against 24.7 us at 23). With two a single pass on 28
-    // to 31 qubits is still up to 3% slower than with 8-byte copies through L1 (644-656 against
-    // 631-647 us at 28), at 27 as fast; most passes run chained. TF32x3 keeps four at every size: up
-    // to 24 qubits they are the faster (55-57 against 57-58 us at 24), beyond that two would be
-    // (332-335 against 359-372 us at 27).
+    // / 351-359 us; from L2 five are faster, 23.4 against 24.7 us at 23). TF32x3 keeps four at every
+    // size: up to 24 qubits they are the faster (55-57 against 57-58 us at 24), beyond that two
+    // would be (332-335 against 359-372 us at 27).
     a.depth = !tf32 && (8ull << n) > (uint64_t(64) << 20) ? 2u : uint32_t(tf32 ? Layout<true>::kSlots : Layout<false>::kSlots);
+    // On large states the loader warps of a CTA drift apart, and the copies of neighbouring units no
+    // longer come together. Starting each unit together, five target sets, us a BF16x3 pass alone and in
+    // step: 31 qubits 5122-5297 and 5061-5177, 29 qubits 1276-1322 and 1269-1297 (8-byte copies
+    // through L1: 4988-5198, 1250-1309); at 28 within 2% either way, at 24 to 27 up to 4% slower. TF32x3
+    // tiles take the SM as long as HBM does, and starting together costs them 20 to 30%.
+    a.step = !tf32 && n >= 29;
     // qubits varying inside a tile: the targets plus the 7 lowest other qubits
     const uint64_t V = tile_qubits(p, n);
     fill_pass(p, n, d_ops, V, &a.pass[0]);

@@ -36,7 +36,9 @@
 //            [Ur; Ui] and [-Ui; Ur] as windows of one [-Ui; Ur; Ui] image per split;
 //   kSub:    the input comes from a compact sub-state (the state is |0> on the qubits
 //            outside it), so the pass also expands that sub-state into the full state;
-//   kChain:  two or three consecutive BF16 passes in one launch, through L2.
+//   kChain:  two or three consecutive BF16 passes in one launch, through L2;
+//   kStep:   a CTA's loader warps start each unit together (single BF16 passes on large states; a
+//            test in the loop of the others cost a 19-qubit circuit 2%).
 //
 // Every wait is bounded (about one second of SM clock); on expiry the kernel raises
 // an error bit, drains its own MMAs and copies, frees its tensor memory and returns.
@@ -86,7 +88,6 @@ struct TcArgs {
     int skip_tile;          // test hook: CTA 0 issues no MMAs for its tile skip_tile (-1: none)
     uint32_t flip;          // XORed into the tile numbers: 0, or tiles - 1 to walk the state backwards
     uint32_t depth;         // slice order: units a loader warp keeps in flight or in conversion, 2..kSlots
-    uint32_t step;          // slice order, BF16, no chain: the CTA's loader warps start each unit together
     // Chain (kChain): see the comment at k_fused_tc.
     int npass;              // passes of the chain, 2..kChainMax
     int clog;               // log2 of the tiles in a chunk
@@ -129,11 +130,12 @@ __device__ __forceinline__ uint32_t swz(uint32_t c) { return c ^ ((c >> 6) & 15u
 // A loader never blocks on a chunk while a tile of its CTA is unconverted, and a wait of
 // (pass p, chunk c) is on (p - 1, c) or (p + 1, c - window) only: with all CTAs resident
 // (a cooperative launch) the schedule cannot deadlock.
-template <bool kStaged, bool kTf32, bool kSub, bool kChain>
+template <bool kStaged, bool kTf32, bool kSub, bool kChain, bool kStep = false>
 __global__ void __launch_bounds__(kChain ? tc::kChainThreads : tc::kThreads, 1)
     k_fused_tc(const __grid_constant__ TcArgs<kChain ? tc::kChainMax : 1> a) {
     static_assert(!(kStaged && kSub), "the sub-state input has a slice-order loader only");
     static_assert(!kChain || (!kStaged && !kSub && !kTf32), "a chain runs BF16 passes in slice order");
+    static_assert(!kStep || (!kStaged && !kSub && !kTf32 && !kChain), "loaders in step: single BF16 passes in slice order");
     using namespace tc;
     constexpr int kThreads = kChain ? tc::kChainThreads : tc::kThreads;
     using L = Layout<kTf32>;
@@ -145,7 +147,7 @@ __global__ void __launch_bounds__(kChain ? tc::kChainThreads : tc::kThreads, 1)
     auto bar_done = [&](int b) { return bar0 + 16u + 8u * uint32_t(b); };
     auto bar_free = [&](int b) { return bar0 + 32u + 8u * uint32_t(b); };
     auto bar_loaded = [&](int b) { return bar0 + 48u + 8u * uint32_t(b); };    // stage b holds the tile's inputs
-    const uint32_t bar_step = bar0 + 48u;  // slice order: the loader warps reached the unit (a.step)
+    const uint32_t bar_step = bar0 + 48u;  // kStep: the loader warps reached the unit
     auto bar_outready = [&](int b) { return bar0 + 64u + 8u * uint32_t(b); };  // stage b holds the tile's outputs
     auto bar_sfree = [&](int b) { return bar0 + 80u + 8u * uint32_t(b); };     // stage b read out by the stores
     // TF32: A is filled and consumed in two K halves (inputs 0..31 by loader warps 0-3,
@@ -558,11 +560,9 @@ __global__ void __launch_bounds__(kChain ? tc::kChainThreads : tc::kThreads, 1)
                 for (int ch = 0; ch < 2; ++ch) {
                     const uint32_t u = 2 * i + uint32_t(ch);
                     __syncwarp();  // every lane has read the slot that is filled next
-                    if constexpr (!kTf32 && !kChain) {
-                        if (a.step) {
-                            if (lane == 0) mbar_arrive(bar_step);
-                            if (!(ok = warp_wait<!kTf32>(bar_step, u & 1u, abort_flag, lim))) break;
-                        }
+                    if constexpr (kStep) {
+                        if (lane == 0) mbar_arrive(bar_step);
+                        if (!(ok = warp_wait<!kTf32>(bar_step, u & 1u, abort_flag, lim))) break;
                     }
                     if (!(ok = top_up(u))) break;
                     const uint32_t later = issued - u - 1;  // units in flight behind this one
@@ -1070,9 +1070,9 @@ void tc_build_ops(const Pass &p, void *host_image, bool tf32) {
     else build_ops_bf16(p, img);
 }
 
-template <bool kStaged, bool kTf32, bool kSub = false, bool kChain = false>
+template <bool kStaged, bool kTf32, bool kSub = false, bool kChain = false, bool kStep = false>
 static int set_smem_attr() {
-    const cudaError_t e = cudaFuncSetAttribute(k_fused_tc<kStaged, kTf32, kSub, kChain>,
+    const cudaError_t e = cudaFuncSetAttribute(k_fused_tc<kStaged, kTf32, kSub, kChain, kStep>,
                                                cudaFuncAttributeMaxDynamicSharedMemorySize, tc::Layout<kTf32>::kAlloc);
     return e == cudaSuccess ? RCS_OK : note_launch_error("tensor-core kernel shared-memory attribute", e);
 }
@@ -1089,6 +1089,7 @@ int tc_prepare_device() {
     if (rc == RCS_OK) rc = set_smem_attr<false, false, true>();
     if (rc == RCS_OK) rc = set_smem_attr<false, true, true>();
     if (rc == RCS_OK) rc = set_smem_attr<false, false, false, true>();
+    if (rc == RCS_OK) rc = set_smem_attr<false, false, false, false, true>();
     if (rc == RCS_OK && dev >= 0 && dev < 64) attr_done[dev] = true;
     return rc;
 }
@@ -1166,7 +1167,7 @@ static int launch_tc(void *psi, int n, const Pass &p, const void *d_ops, int *d_
     // step: 31 qubits 5122-5297 and 5061-5177, 29 qubits 1276-1322 and 1269-1297 (8-byte copies
     // through L1: 4988-5198, 1250-1309); at 28 within 2% either way, at 24 to 27 up to 4% slower. TF32x3
     // tiles take the SM as long as HBM does, and starting together costs them 20 to 30%.
-    a.step = !tf32 && n >= 29;
+    const bool step = !tf32 && !staged && !sub && n >= 29;
     // qubits varying inside a tile: the targets plus the 7 lowest other qubits
     const uint64_t V = tile_qubits(p, n);
     fill_pass(p, n, d_ops, V, &a.pass[0]);
@@ -1187,7 +1188,8 @@ static int launch_tc(void *psi, int n, const Pass &p, const void *d_ops, int *d_
     } else if (tf32) {
         kernel = staged ? k_fused_tc<true, true, false, false> : k_fused_tc<false, true, false, false>;
     } else {
-        kernel = staged ? k_fused_tc<true, false, false, false> : k_fused_tc<false, false, false, false>;
+        kernel = staged ? k_fused_tc<true, false, false, false>
+                 : step ? k_fused_tc<false, false, false, false, true> : k_fused_tc<false, false, false, false>;
     }
     const cudaError_t e = launch_after(kernel, grid, kThreads, smem, st, a);
     return e == cudaSuccess ? RCS_OK : note_launch_error("tensor-core pass", e);

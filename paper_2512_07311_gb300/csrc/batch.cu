@@ -94,17 +94,18 @@ struct BArgs {
 // slice these reads (one per 4) bound the kernel at width 4, 28 TFLOP/s; two slices' inputs
 // fit the registers up to width 4. An item without a second slice for its threads is worked on
 // one by one: the multiply-adds of a slice that is not there cost 48 circuits of 8 to 12 qubits
-// at width 4 16 to 24% (12 qubits 117 against 142 us). At width 5 the whole mat-vec in a row is
-// 64 KB of code, which with the other widths' no longer fits the instruction cache: two rows at
-// a time take 65 us instead of 92 for 48 circuits of 8 qubits (80 before the code for two
-// slices), 790 instead of 830 (800) at 15 and 3.15 instead of 3.24 ms (3.27) for 12 of 20. offs:
-// the 2^K target offsets in shared memory, read back through a volatile pointer at each use so
-// they are not held in registers across the mat-vec.
+// at width 4 16 to 24% (12 qubits 117 against 142 us); their code stays out of line, so that the
+// loops that large circuits run stay as they are. At width 5 the whole mat-vec in a row is 64 KB
+// of code, which with the other widths' no longer fits the instruction cache: four rows at a time
+// take 71 us instead of 92 for 48 circuits of 8 qubits (80 before the code for two slices), 811
+// instead of 826 (797) at 15 and 3.11 instead of 3.23 ms (3.28) for 12 of 20. offs: the 2^K target
+// offsets in shared memory, read back through a volatile pointer at each use so they are not held
+// in registers across the mat-vec.
 template <int K, int kPer>
 __device__ __forceinline__ void apply_items(float2 *__restrict__ psi, const int *t, const float4 *sU,
                                             const volatile uint64_t *offs, uint64_t s_begin, uint64_t s_end) {
     constexpr int D = 1 << K;
-    constexpr int kRows = K == 5 ? 2 : D;  // rows of U in the code at once
+    constexpr int kRows = K == 5 ? 4 : D;  // rows of U in the code at once
 #pragma unroll 1
     for (uint64_t s = s_begin + threadIdx.x; s < s_end; s += uint64_t(kPer) * kThreads) {
         float2 *p[kPer];
@@ -143,6 +144,17 @@ __device__ __forceinline__ void apply_items(float2 *__restrict__ psi, const int 
             __stcg(p[0] + o, acc[0]);
             if (both) __stcg(p[kPer - 1] + o, acc[kPer - 1]);
         }
+    }
+}
+
+// An item of at most kThreads slices at width 1 to 4.
+__device__ __noinline__ void apply_single(int k, float2 *__restrict__ psi, const int *t, const float4 *sU,
+                                          const volatile uint64_t *offs, uint64_t s_begin, uint64_t s_end) {
+    switch (k) {
+        case 1: apply_items<1, 1>(psi, t, sU, offs, s_begin, s_end); break;
+        case 2: apply_items<2, 1>(psi, t, sU, offs, s_begin, s_end); break;
+        case 3: apply_items<3, 1>(psi, t, sU, offs, s_begin, s_end); break;
+        default: apply_items<4, 1>(psi, t, sU, offs, s_begin, s_end); break;
     }
 }
 
@@ -229,13 +241,16 @@ __global__ void __launch_bounds__(kThreads, 2) k_batch_apply(const __grid_consta
         int t[kMaxK];
 #pragma unroll
         for (int i = 0; i < kMaxK; ++i) t[i] = ps.t[i];
-        const bool two = s1 > s0 + kThreads;
-        switch (ps.k) {
-            case 1: two ? apply_items<1, 2>(in.psi, t, sU, sOff, s0, s1) : apply_items<1, 1>(in.psi, t, sU, sOff, s0, s1); break;
-            case 2: two ? apply_items<2, 2>(in.psi, t, sU, sOff, s0, s1) : apply_items<2, 1>(in.psi, t, sU, sOff, s0, s1); break;
-            case 3: two ? apply_items<3, 2>(in.psi, t, sU, sOff, s0, s1) : apply_items<3, 1>(in.psi, t, sU, sOff, s0, s1); break;
-            case 4: two ? apply_items<4, 2>(in.psi, t, sU, sOff, s0, s1) : apply_items<4, 1>(in.psi, t, sU, sOff, s0, s1); break;
-            default: apply_items<5, 1>(in.psi, t, sU, sOff, s0, s1); break;
+        if (ps.k <= 4 && s1 <= s0 + kThreads) {
+            apply_single(ps.k, in.psi, t, sU, sOff, s0, s1);
+        } else {
+            switch (ps.k) {
+                case 1: apply_items<1, 2>(in.psi, t, sU, sOff, s0, s1); break;
+                case 2: apply_items<2, 2>(in.psi, t, sU, sOff, s0, s1); break;
+                case 3: apply_items<3, 2>(in.psi, t, sU, sOff, s0, s1); break;
+                case 4: apply_items<4, 2>(in.psi, t, sU, sOff, s0, s1); break;
+                default: apply_items<5, 1>(in.psi, t, sU, sOff, s0, s1); break;
+            }
         }
         __syncthreads();
         if (threadIdx.x == 0 && (long long)s_item != a.skip_item) {
